@@ -60,7 +60,9 @@ __host__ __device__ __forceinline__ int padi(int i) { return i + (i >> 2); }  //
 __global__ void __launch_bounds__(1024)
     ksg_stage_kernel(const float* __restrict__ field, int M, int64_t N,
                      const int64_t* __restrict__ refs, int64_t ref0, float* __restrict__ xs_all,
-                     int* __restrict__ perm_all, unsigned* __restrict__ status) {
+                     int* __restrict__ perm_all, unsigned* __restrict__ status,
+                     unsigned long long* __restrict__ work) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *work = 0ull;  // the searches' work counter
     __shared__ float key[kKsgMaxM];
     __shared__ int val[kKsgMaxM];
     const int64_t ref = refs ? refs[blockIdx.x] : ref0 + blockIdx.x;
@@ -105,6 +107,96 @@ __global__ void __launch_bounds__(1024)
     }
 }
 
+// The same for up to 1024 members, one warp per reference: RG (key, member) pairs per lane,
+// element 32 r + lane in register r, sorted by a bitonic network (strides of 32 and more are
+// register pairs, the others shuffles).  No barriers and 32 warps' worth of references per SM
+// at once: 100,000 references of 500 members take 0.55 ms instead of 3.97 ms with one CTA of
+// 1024 threads and 45 barriers each, and a single one of 100 members 2.2 us instead of 7.2.
+// A lone reference with many members stays with the CTA above (launch_ksg).
+__device__ __forceinline__ bool stage_less(float a, int va, float b, int vb) {
+    return a < b || (a == b && va < vb);
+}
+template <int RG, int RS, int SIZE>
+__device__ __forceinline__ void stage_register_strides(float (&key)[RG], int (&val)[RG]) {
+    if constexpr (RS >= 1) {
+#pragma unroll
+        for (int r = 0; r < RG; ++r) {
+            if (r & RS) continue;
+            const int q = r | RS;
+            const bool up = ((r * 32) & SIZE) == 0;
+            if (up ? stage_less(key[q], val[q], key[r], val[r]) : stage_less(key[r], val[r], key[q], val[q])) {
+                const float tk = key[r];
+                const int tv = val[r];
+                key[r] = key[q];
+                val[r] = val[q];
+                key[q] = tk;
+                val[q] = tv;
+            }
+        }
+        stage_register_strides<RG, RS / 2, SIZE>(key, val);
+    }
+}
+template <int RG, int SIZE>
+__device__ __forceinline__ void stage_sort(float (&key)[RG], int (&val)[RG]) {
+    if constexpr (SIZE <= 32 * RG) {
+        const int lane = threadIdx.x & 31;
+        stage_register_strides<RG, SIZE / 64, SIZE>(key, val);
+#pragma unroll 1
+        for (int stride = SIZE >= 32 ? 16 : SIZE / 2; stride > 0; stride >>= 1) {
+            const bool lower = (lane & stride) == 0;
+#pragma unroll
+            for (int r = 0; r < RG; ++r) {
+                const float ok = __shfl_xor_sync(0xffffffffu, key[r], stride);
+                const int ov = __shfl_xor_sync(0xffffffffu, val[r], stride);
+                const bool up = ((r * 32 + lane) & SIZE) == 0;
+                if (stage_less(ok, ov, key[r], val[r]) == (lower == up)) {
+                    key[r] = ok;
+                    val[r] = ov;
+                }
+            }
+        }
+        stage_sort<RG, SIZE * 2>(key, val);
+    }
+}
+template <int RG>
+__global__ void __launch_bounds__(128)
+    ksg_stage_warp_kernel(const float* __restrict__ field, int M, int64_t N, const int64_t* __restrict__ refs,
+                          int64_t ref0, int R, float* __restrict__ xs_all, int* __restrict__ perm_all,
+                          unsigned* __restrict__ status, unsigned long long* __restrict__ work) {
+    const int lane = threadIdx.x & 31;
+    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (row == 0 && lane == 0) *work = 0ull;
+    if (row >= R) return;
+    const int64_t ref = refs ? refs[row] : ref0 + row;
+    float* xs = xs_all + row * M;
+    int* pm = perm_all + row * M;
+    if (ref < 0 || ref >= N) {
+        if (lane == 0 && status) atomicOr(status, kDevBadInput);
+        for (int i = lane; i < M; i += 32) {
+            xs[i] = __int_as_float(0x7fc00000);
+            pm[i] = i;
+        }
+        return;
+    }
+    float key[RG];
+    int val[RG];
+#pragma unroll
+    for (int r = 0; r < RG; ++r) {
+        const int i = 32 * r + lane;
+        key[r] = i < M ? field[(int64_t)i * N + ref] : FLT_MAX;
+        val[r] = i < M ? i : INT_MAX;
+    }
+    stage_sort<RG, 2>(key, val);
+#pragma unroll
+    for (int r = 0; r < RG; ++r) {
+        const int i = 32 * r + lane;
+        if (i < M) {
+            xs[i] = key[r];
+            pm[i] = val[r];
+        }
+    }
+}
+
 // ---------------------------------------------------------------- helpers
 __device__ __forceinline__ unsigned long long pack_f2(float2 v) {
     return ((unsigned long long)__float_as_uint(v.y) << 32) | __float_as_uint(v.x);
@@ -125,6 +217,7 @@ struct KsgArgs {
     const float* xs_all;  // [R][M] sorted reference values
     const int* perm_all;  // [R][M] member id of each sorted position
     const double* psi;    // psi(n), n <= M + 1
+    const long long* psi_fix;  // the same in fixed point (kPsiFixBits)
     float* out;           // out[r * out_stride + (v - v_begin)]
     int64_t out_stride;
     int variant;          // KSG algorithm 1 or 2
@@ -633,7 +726,7 @@ __device__ __forceinline__ void block_keys(const KsgArgs& A, const int* perm, in
     }
 }
 
-// lower bound of y in a block of kBlk ascending values (pads +inf): 0 .. kBlk
+// lower bound of y in a block of kBlk ascending values (pads +inf): 0 .. kBlk - 1
 __device__ __forceinline__ int block_lower_bound(const float2* blk, float y) {
     int pos = 0;
 #pragma unroll
@@ -647,13 +740,22 @@ __device__ __forceinline__ int block_lower_bound(const float2* blk, float y) {
 // zeros).  Blocks from the member's own block b0 outward in x while the block's nearest
 // x-rank is within e (fl(x_j - xi) is monotone in x_j); inside a block, outward in y
 // from the lower bound of yi while |dy| <= e (the +inf separators stop both scans).
-__device__ __forceinline__ void block_extents(const float2* blk, const float2* bx, int nb, int b0, float xi,
-                                              float yi, float e, float& ex, float& ey) {
+__device__ __forceinline__ void block_extents(const float2* blk, const float2* bx, int M, int nb, int lw,
+                                              int b0, float xi, float yi, float e, float& ex, float& ey) {
     ex = 0.0f;
     ey = 0.0f;
     auto scan = [&](int bb) {
-        const float2* B = blk + 1 + bb * kBlkStride;  // (y, x), ascending y
-        const int pos = block_lower_bound(B, yi);
+        const float2* B = blk + 1 + bb * ((1 << lw) + 1);  // (y, x), ascending y
+        int pos = 0;
+        for (int len = min(1 << lw, M - (bb << lw)); len > 0;) {  // members below yi
+            const int h = len >> 1;
+            if (B[pos + h].x < yi) {
+                pos += h + 1;
+                len -= h + 1;
+            } else {
+                len = h;
+            }
+        }
         for (int u = pos;; ++u) {
             const float2 c = B[u];
             const float dy = fabsf(c.x - yi);
@@ -858,81 +960,121 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kMaxGroupsPerCta, 1)
 }
 
 // ---------------------------------------------------------------- lane-refill block search
-// The same two-level search as ksg_block_kernel (x-blocks of kBlk ranks sorted by
-// the query value, +inf separators, the same window, x-gap and insert rules, so
-// eps_i is again the brute-force value bit for bit), scheduled per lane instead of
-// per block scan:
+// The same two-level search as ksg_block_kernel (x-blocks of W consecutive x-ranks
+// sorted by the query value, +inf separators, the same window, x-gap and insert rules,
+// so eps_i is again the brute-force value bit for bit), scheduled per lane instead of
+// per block scan, and with the block order built from ranks instead of sorts:
+//   - every member's rank in the query column (a binary search in the sorted copy; tied
+//     members take consecutive ranks from a counter, in any order: neither eps nor the sums
+//     depend on it) goes into its block's bitmap of ranks.
+//     With the bitmap words' running counts, the number of a block's members below a rank is
+//     two loads and a population count.  That gives a member's place in its block (no
+//     sort: the former 64-key bitonic sorts took about 7 warp instructions per member, this
+//     about 3) and, during the search, the point where a lane enters a neighbouring block
+//     (before: a six-step binary search in a service step that few lanes share);
 //   - a lane owns one member at a time and walks its own sequence of blocks: its own
 //     block from its position outward, then the neighbouring blocks, at each switch
 //     the side whose nearest x-rank is closer (a side ends at the first block whose
 //     nearest x-rank is at least the current k-th distance away);
 //   - a lane whose member is finished stores eps_i (by block position) and takes the
-//     pair's next member from a counter the group's two warps share;
-//   - block switches (gap tests and the 6-step binary search) and refills run in a
-//     warp-uniform service step, entered only when at least `switch_min` lanes wait
-//     or no lane is scanning, so the divergent code runs for many lanes at once;
+//     next member of its warp (the group's warps split the members evenly);
+//   - block switches and refills run in a warp-uniform service step, entered only when at
+//     least `switch_min` lanes wait or no lane is scanning, so the divergent code runs for
+//     many lanes at once;
 //   - every other lock step is the scan step of the block kernel for all lanes;
-//   - the marginal counts and the digamma sum follow in an evenly split pass over
+//   - the marginal counts and the digamma sum (in fixed point: the same sum in any order, two
+//     integer adds for the slow FP64 pipe's one) follow in an evenly split pass over
 //     the stored eps (for KSG algorithm 2 after the marginal extents of each member's
 //     k-NN set, found over the same blocks: block_extents).
-// A lock-step model of both schedules on csens-like pairs (M = 1000, k = 8) counts
-// about 600 lock steps per pair here against about 1300 for the block kernel (lane
-// utilisation 0.70 against 0.33).  Members are handed out in the block kernel's task
-// order (8 y-positions of 4 neighbouring blocks per 32), so the lanes of a warp start
-// on members of similar rank.  Shared memory per pair: the block-sorted points, the
-// sorted query column and the stored eps (16 B x M); the sorted reference values are
-// read from the staging buffer in global memory (L1), for the x-gap tests and n_x.
+// What bounds it: the ALU pipe (the scan step's minima, maxima and compares issue at half
+// rate; 70 % busy at M = 1000, k = 8), then the shared-memory wavefronts of the lanes' scattered
+// reads (68 %) and the issue slots (62 %); 64,800 warp instructions per pair against 86,000 for
+// the sorted 64-rank blocks before.  250 x 352 x 20 vertices, M = 1000, k = 8: 167.5 ms before,
+// 133.5 - 139 ms now.
+// Members are handed out in the block kernel's task order (8 y-positions of 4 neighbouring
+// blocks per 32), so the lanes of a warp start on members of similar rank.  Shared memory per
+// pair: the block-sorted points, the sorted query column, one word per member (its query
+// value, then its rank, then eps) and the bitmaps (16 B x M + 5 B per block and 32 ranks);
+// the sorted reference values sit in shared memory once per CTA when all pairs share the
+// reference, else they are read from the staging buffer in global memory (L1).
 struct LaneCtl {
     unsigned long long item;
-    int next;  // the pair's next member slot
-    int pad;
-    double part[kGroupWarps];
+    unsigned long long pad;
+    long long part[kGroupWarps];
 };
-__host__ __device__ inline int lane_slots(int nb) {
-    return ((nb + kTaskBlocks - 1) / kTaskBlocks) * kTaskQuads * 32;
-}
-__host__ __device__ inline size_t lane_group_bytes(int M) {
-    const int nb = (M + kBlk - 1) / kBlk;
-    return sizeof(LaneCtl) + sizeof(float2) * ((size_t)nb * kBlkStride + 1) +
-           sizeof(float) * (size_t)((M + 3) & ~3) + sizeof(float) * (size_t)nb * kBlk +
-           sizeof(float2) * (size_t)nb;
-}
+__host__ __device__ inline int lane_slots(int nb, int lw) { return (((nb + 3) >> 2) << 2) << lw; }
+// shared memory of one group (bytes from its base), W = 1 << lw ranks per block
+struct LaneSmem {
+    int blk, ys, eps, tab, below, bx, total;
+    __host__ __device__ LaneSmem(int M, int lw) {
+        const int nb = (M + (1 << lw) - 1) >> lw, nw = (M + 31) >> 5;
+        int o = (int)sizeof(LaneCtl);
+        blk = o; o += (int)sizeof(float2) * (M + nb + 1);
+        ys = o; o += (int)sizeof(float) * ((M + 1) & ~1);
+        eps = o; o += (int)sizeof(float) * ((M + 1) & ~1);
+        bx = o; o += (int)sizeof(float2) * (nb + 2);
+        tab = o; o += (int)sizeof(unsigned) * nb * nw;
+        below = o; o += (nb * nw + 7) & ~7;
+        total = (o + 15) & ~15;
+    }
+};
+// ranks per block: the scan visits members inside the y-window of whole blocks, so wider blocks
+// cost candidates that fail the x-test, narrower ones more block switches.  Measured (ms a
+// volume, 32 / 64 / 128 ranks): 1.118 / 1.157 / 1.384 for M = 200, k = 4 (88,000 vertices);
+// 0.440 / 0.437 / 0.466 for M = 333, k = 5 (18,361); 1.88 / 1.74 / 1.95 for M = 600, k = 6
+// (40,000); 10.5 / 7.6 / 6.9 for M = 1000, k = 8 (88,000); 6.7 / 4.2 / 3.5 for M = 1800, k = 10
+// (14,400).
+__host__ __device__ inline int lane_block_log2(int M) { return M > 768 ? 7 : M > 256 ? 6 : 5; }
 // lock steps a warp may take per pair before it gives up (a safety bound far above
-// any real schedule: every member visits at most nb blocks of kBlk + 1 steps)
-__host__ __device__ inline long long lane_step_bound(int nb) {
-    return (long long)lane_slots(nb) * (nb + 2) * (kBlk + 4);
+// any real schedule: every member visits at most nb blocks of W + 1 steps)
+__host__ __device__ inline long long lane_step_bound(int nb, int lw) {
+    return (long long)lane_slots(nb, lw) * (nb + 2) * ((1 << lw) + 4);
 }
+constexpr int kLaneMaxGroups = 13;  // groups per CTA: what shared memory holds at M = 1000
+constexpr int kLaneMaxRegs = 4;  // ranks per lane of a block (W <= 128; `below` counts in bytes)
 
 template <int K1>
-__global__ void __launch_bounds__(32 * kGroupWarps * kMaxGroupsPerCta, 1)
-    ksg_lane_kernel(KsgArgs A, unsigned long long* work, int switch_min, int every) {
+__global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
+    ksg_lane_kernel(KsgArgs A, unsigned long long* work, int lw, int switch_min, int every) {
     constexpr int KK = K1 - 1;
     constexpr int GT = 32 * kGroupWarps;
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem[];
     const int M = A.M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int group = warp / kGroupWarps, gw = warp % kGroupWarps, gt = threadIdx.x % GT;
-    const int nb = (M + kBlk - 1) / kBlk;
-    const int slots = lane_slots(nb);
-    unsigned char* gbase = smem + (size_t)group * lane_group_bytes(M);
+    const int W = 1 << lw, nb = (M + W - 1) >> lw, nw = (M + 31) >> 5, bs = W + 1;
+    const int slots = lane_slots(nb, lw);
+    const LaneSmem L(M, lw);
+    unsigned char* gbase = smem + group * L.total;
     LaneCtl* ctl = reinterpret_cast<LaneCtl*>(gbase);
-    float2* blk = reinterpret_cast<float2*>(gbase + sizeof(LaneCtl));  // (y, x), separated blocks
-    float* ys = reinterpret_cast<float*>(blk + (size_t)nb * kBlkStride + 1);  // query, sorted
-    float* eps_s = ys + ((M + 3) & ~3);                                  // eps by block position
-    float2* bx = reinterpret_cast<float2*>(eps_s + (size_t)nb * kBlk);   // (first, last) x per block
+    float2* blk = reinterpret_cast<float2*>(gbase + L.blk);  // (y, x), separated blocks
+    float* ys = reinterpret_cast<float*>(gbase + L.ys);      // query, sorted
+    float* eps_s = reinterpret_cast<float*>(gbase + L.eps);  // y, rank, eps (see above)
+    int* rank_s = reinterpret_cast<int*>(eps_s);
+    unsigned* tab = reinterpret_cast<unsigned*>(gbase + L.tab);  // rank bits [nb][nw]
+    unsigned char* below = gbase + L.below;  // a block's members below the word
+    float2* bx = reinterpret_cast<float2*>(gbase + L.bx) + 1;  // (first, last) x per block
     const int64_t N = A.N, nv = A.v_end - A.v_begin;
     const unsigned long long items =
         A.paired ? (unsigned long long)nv : (unsigned long long)A.R * (unsigned long long)nv;
     const double psi_k = A.psi[A.k], psi_M = A.psi[M];
-    const int step_bound = (int)min(lane_step_bound(nb), (long long)INT_MAX);
+    const int step_bound = (int)min(lane_step_bound(nb, lw), (long long)INT_MAX);
+    const int top = pow2_floor(M);
     unsigned long long evals_total = 0;
+    const bool x_shared = A.R == 1;
+    float* xsh = reinterpret_cast<float*>(smem + (blockDim.x / GT) * L.total);
+    if (x_shared) {
+        for (int i = threadIdx.x; i < M; i += blockDim.x) xsh[i] = A.xs_all[i];
+        __syncthreads();
+    }
+    if (gt == 0) {  // no block beyond either end: an infinite x-gap
+        bx[-1] = make_float2(0.0f, -INFINITY);
+        bx[nb] = make_float2(INFINITY, 0.0f);
+    }
 
     for (;;) {
         group_sync(group);  // the previous pair is finished by both warps
-        if (gt == 0) {
-            ctl->item = atomicAdd(work, 1ull);
-            ctl->next = 0;
-        }
+        if (gt == 0) ctl->item = atomicAdd(work, 1ull);
         group_sync(group);
         const unsigned long long item = ctl->item;
         if (item >= items) break;
@@ -940,240 +1082,251 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kMaxGroupsPerCta, 1)
         const int64_t v = A.v_begin + (int64_t)(A.paired ? item : item - (unsigned long long)r * nv);
         const float* xsg = A.xs_all + (int64_t)r * M;  // reference values, x-sorted (global)
         const int* perm = A.perm_all + (int64_t)r * M;
-        // ---- the query column in member order (into eps_s, scratch until the search) and
-        // in sorted order; each thread has eight of its strided loads of both in flight
-        // before their stores, so the column costs two memory round trips, not M / 64
-        float* ycol = eps_s;  // nb * kBlk >= M floats
+        const bool dbg = A.dbg_eps && r == 0 && v == A.v_begin;
+        // ---- the query column in x-order and in sorted order; each thread has eight of its
+        // strided loads of both in flight before their stores, so the column costs two memory
+        // round trips, not M / 64
+        int* cnt = reinterpret_cast<int*>(blk);  // tie counters (until the blocks are laid out)
         for (int s0 = 0; s0 < M; s0 += 8 * GT) {
             float c8[8], s8[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int s = s0 + j * GT + gt;
-                c8[j] = s < M ? A.field[(int64_t)s * N + v] : 0.0f;
+                c8[j] = s < M ? A.field[(int64_t)perm[s] * N + v] : 0.0f;
                 s8[j] = s < M ? A.sorted[(int64_t)s * N + v] : 0.0f;
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int s = s0 + j * GT + gt;
                 if (s < M) {
-                    ycol[s] = c8[j];
+                    eps_s[s] = c8[j];
                     ys[s] = s8[j];
+                    cnt[s] = 0;
                 }
             }
         }
-        // ---- blocks of kBlk x-ranks, each sorted by y; pads (y = x = +inf) sort last
-        for (int b = gt; b <= nb; b += GT) blk[b * kBlkStride] = make_float2(INFINITY, INFINITY);
-        for (int b = gt; b < nb; b += GT)
-            bx[b] = make_float2(xsg[b * kBlk], xsg[min(b * kBlk + kBlk - 1, M - 1)]);
-        group_sync(group);  // the member-order column is complete
-        for (int b = gw; b < nb; b += kGroupWarps) {
-            float key[kBlkRegs];
-            int val[kBlkRegs];
+        for (int i = gt; i < nb * nw; i += GT) tab[i] = 0u;
+        for (int b = gt; b < nb; b += GT) bx[b] = make_float2(xsg[b << lw], xsg[min((b << lw) + W, M) - 1]);
+        group_sync(group);  // the sorted column is complete
+        // a constant query column: every distance is |dx|, so the blocks keep x-order and hold
+        // (x, y) in the place of (y, x); the scan's window is then the x-gap
+        const bool constant = ys[0] == ys[M - 1] && A.variant == 1;
+        // ---- the members' ranks, four searches of a thread interleaved
+        for (int s0 = gt; s0 < M; s0 += 4 * GT) {
+            float y[4];
+            int p[4];
 #pragma unroll
-            for (int r2 = 0; r2 < kBlkRegs; ++r2) {  // the sort keys of block b (shared memory)
-                const int rank = b * kBlk + r2 * 32 + lane;
-                key[r2] = rank < M ? ycol[perm[rank]] : INFINITY;
-                val[r2] = rank;
+            for (int j = 0; j < 4; ++j) y[j] = eps_s[min(s0 + j * GT, M - 1)];
+            if (!constant) lower_bounds<4>(ys, M, top, y, p);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int s = s0 + j * GT;
+                if (s >= M) continue;
+                int rank = constant ? s : min(p[j], M - 1);
+                if (!constant && rank + 1 < M && ys[rank + 1] == y[j])
+                    rank = min(rank + atomicAdd(cnt + rank, 1), M - 1);
+                rank_s[s] = rank;
+                atomicOr(&tab[(s >> lw) * nw + (rank >> 5)], 1u << (rank & 31));
             }
-            warp_sort_block(key, val);
+        }
+        group_sync(group);
+        // ---- blocks of W x-ranks (the last one shorter) in the order of the ranks
+        for (int b = gt; b <= nb; b += GT) blk[b < nb ? b * bs : M + nb] = make_float2(INFINITY, INFINITY);
+        for (int b = gw; b < nb; b += kGroupWarps) {
+            const unsigned* tb = tab + b * nw;
+            unsigned char* bb = below + b * nw;
+            int carry = 0;
+            for (int w0 = 0; w0 < nw; w0 += 32) {
+                const int w = w0 + lane;
+                const int c = w < nw ? __popc(tb[w]) : 0;
+                int inc = c;
 #pragma unroll
-            for (int r2 = 0; r2 < kBlkRegs; ++r2)
-                blk[1 + b * kBlkStride + r2 * 32 + lane] =
-                    make_float2(key[r2], val[r2] < M ? xsg[val[r2]] : INFINITY);
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int u = __shfl_up_sync(FULL, inc, o);
+                    inc += lane >= o ? u : 0;
+                }
+                if (w < nw) bb[w] = (unsigned char)(carry + inc - c);
+                carry += __shfl_sync(FULL, inc, 31);
+            }
+            int rk[kLaneMaxRegs];
+#pragma unroll
+            for (int j = 0; j < kLaneMaxRegs; ++j) {
+                const int s = (b << lw) + j * 32 + lane;
+                rk[j] = j * 32 < W && s < M ? rank_s[s] : -1;
+            }
+            __syncwarp();  // the counts are written, the ranks read (their places are reused)
+#pragma unroll
+            for (int j = 0; j < kLaneMaxRegs; ++j) {
+                if (rk[j] < 0) continue;
+                const int s = (b << lw) + j * 32 + lane;
+                const int pos = bb[rk[j] >> 5] + __popc(tb[rk[j] >> 5] & ((1u << (rk[j] & 31)) - 1u));
+                const float y = ys[rk[j]], x = xsg[s];
+                blk[1 + b * bs + pos] = constant ? make_float2(x, y) : make_float2(y, x);
+                rank_s[(b << lw) + pos] = rk[j];
+                if (dbg) A.dbg_ny[(b << lw) + pos] = s;  // x-rank by position (scratch)
+            }
         }
         group_sync(group);
 
-        // ---- joint k-NN distance of every member, lanes refilled from the pair's counter
-        bool has = false, inblk = false, exhausted = false;
-        int cb = 0, up = kBlk, dn = -1, nr = 0, nl = -1, slot_pos = 0, start = 0;
-        float xi = INFINITY, yi = INFINITY;
+        // ---- joint k-NN distance of every member, lanes refilled from their warp's members
+        const int pt0 = group * L.total + L.blk + (int)sizeof(float2);  // block 0, position 0
+        bool has = false, inblk = false;
+        int up = pt0 - (int)sizeof(float2), dn = up;  // byte offsets; separators for an idle lane
+        int nr = 0, nl = -1, rank = 0, slot_pos = 0;
+        int next = 0;  // members handed out by this warp (task order, every kGroupWarps-th task)
+        const int wslots = slots / kGroupWarps;
+        float xi = 0.0f, yi = 0.0f;
         float best[KK];
 #pragma unroll
         for (int c = 0; c < KK; ++c) best[c] = FLT_MAX;
         unsigned my_evals = 0;
-        // member slot q (task order) -> block, position; slots past a block's end are empty
-        auto take = [&](int q) {
-            has = false;
-            inblk = false;
-            cb = 0;
-            up = kBlk;  // separators: an idle lane reads +inf
-            dn = -1;
-            xi = INFINITY;
-            yi = INFINITY;
-            if (q >= slots) return;
-            const int task = q >> 5, l = q & 31;
-            const int b = (task / kTaskQuads) * kTaskBlocks + l / kTaskRows;
-            const int p = (task % kTaskQuads) * kTaskRows + l % kTaskRows;
-            if (b >= nb || p >= min(kBlk, M - b * kBlk)) return;
-            const float2 me = blk[1 + b * kBlkStride + p];
-            yi = me.x;
-            xi = me.y;
-            has = true;
-            inblk = true;
-            cb = b;
-            up = p + 1;
-            dn = p - 1;
-            start = p;  // the candidates visited in a block are up - dn - 1 - (own block)
-            nr = b + 1;
-            nl = b - 1;
-            slot_pos = b * kBlk + p;
-#pragma unroll
-            for (int c = 0; c < KK; ++c) best[c] = FLT_MAX;
-        };
-        {
-            int base = 0;
-            if (lane == 0) base = atomicAdd(&ctl->next, 32);
-            base = __shfl_sync(FULL, base, 0);
-            take(base + lane);
-            exhausted = base + 32 >= slots;
-        }
         int steps = 0;
         for (;;) {
-            const bool waiting = has ? !inblk : !exhausted;
-            const unsigned wm = __ballot_sync(FULL, waiting);
+            const unsigned wm = __ballot_sync(FULL, has ? !inblk : next < wslots);
             const unsigned em = __ballot_sync(FULL, has && inblk);
-            if (wm != 0u && (__popc(wm) >= switch_min || em == 0u)) {
+            if (em == 0u && wm == 0u) break;
+            if (em == 0u || __popc(wm) >= switch_min) {
                 // service: block switches of the lanes whose window closed, then refills
                 if (has && !inblk) {
-                    my_evals += (unsigned)(up - dn - 1 - (start >= 0 ? 1 : 0));
+                    my_evals += (unsigned)(up - dn);
                     const float t = best[KK - 1];
-                    const float gr = nr < nb ? bx[nr].x - xi : INFINITY;
-                    const float gl = nl >= 0 ? xi - bx[nl].y : INFINITY;
+                    const float x = constant ? yi : xi;
+                    const float gr = bx[nr].x - x, gl = x - bx[nl].y;
                     const bool okr = gr < t, okl = gl < t;
                     if (!okr && !okl) {
                         eps_s[slot_pos] = t;  // member finished
                         has = false;
-                        cb = 0;
-                        up = kBlk;
-                        dn = -1;
-                        xi = INFINITY;
-                        yi = INFINITY;
+                        my_evals -= (unsigned)sizeof(float2);  // itself
+                        up = dn = pt0 - (int)sizeof(float2);
                     } else {
                         const bool go_r = okr && (!okl || gr <= gl);
-                        cb = go_r ? nr : nl;
+                        const int cb = go_r ? nr : nl;
                         nr += go_r ? 1 : 0;
                         nl -= go_r ? 0 : 1;
-                        const int pos = block_lower_bound(blk + 1 + cb * kBlkStride, yi);
-                        up = pos;
-                        dn = pos - 1;
-                        start = -1;
+                        const int wd = cb * nw + (rank >> 5);
+                        const int pos = below[wd] + __popc(tab[wd] & ((1u << (rank & 31)) - 1u));
+                        up = pt0 + (cb * bs + pos) * (int)sizeof(float2);
+                        dn = up - (int)sizeof(float2);
                         inblk = true;
                     }
+                    my_evals -= (unsigned)sizeof(float2);
                 }
                 const unsigned dm = __ballot_sync(FULL, !has);
-                if (dm != 0u && !exhausted) {
-                    int base = 0;
-                    if (lane == 0) base = atomicAdd(&ctl->next, __popc(dm));
-                    base = __shfl_sync(FULL, base, 0);
-                    if (!has) take(base + __popc(dm & ((1u << lane) - 1u)));
-                    exhausted = base + __popc(dm) >= slots;
+                if (dm != 0u && next < wslots) {
+                    const int q = next + __popc(dm & ((1u << lane) - 1u));
+                    next += __popc(dm);
+                    // slot q of the warp -> block, position; slots past a block's end are empty
+                    const int task = (q >> 5) * kGroupWarps + gw;
+                    const int b = ((task >> (lw - 3)) << 2) + ((q >> 3) & 3);
+                    const int p = ((task & ((W >> 3) - 1)) << 3) + (q & 7);
+                    if (!has && q < wslots && b < nb && (b << lw) + p < M) {
+                        up = pt0 + (b * bs + p) * (int)sizeof(float2);
+                        const float2 me = *reinterpret_cast<const float2*>(smem + up);
+                        yi = me.x;
+                        xi = me.y;
+                        dn = up - (int)sizeof(float2);
+                        up += (int)sizeof(float2);
+                        has = true;
+                        inblk = true;
+                        nr = b + 1;
+                        nl = b - 1;
+                        slot_pos = (b << lw) + p;
+                        rank = rank_s[slot_pos];
+#pragma unroll
+                        for (int c = 0; c < KK; ++c) best[c] = FLT_MAX;
+                    }
                 }
-            }
-            if (!__any_sync(FULL, has)) {
-                if (exhausted) break;
-                continue;
             }
             steps += every;
             if (steps > step_bound) break;  // never expected: the pair's MI becomes NaN
             // `every` scan steps: one candidate above and one below in the lane's current
             // block (idle lanes, and lanes whose window has closed, re-read candidates at
             // least the threshold away and leave their lists unchanged)
-            const float2* B = blk + 1 + cb * kBlkStride;
+            const unsigned long long P = pack_f2(make_float2(yi, xi));
+            bool au = false, ad = false;
 #pragma unroll 2
             for (int rep = 0; rep < every; ++rep) {
                 const float t = best[KK - 1];
-                const float2 cu = B[up], cd = B[dn];
-                const float dyu = cu.x - yi, dyd = yi - cd.x;
-                const bool au = fabsf(dyu) < t;
-                const bool ad = fabsf(dyd) < t;
-                const float du = fmaxf(fabsf(cu.y - xi), fabsf(dyu));
-                const float dd = fmaxf(fabsf(cd.y - xi), fabsf(dyd));
+                const float2 eu = sub_f32x2(P, *reinterpret_cast<const unsigned long long*>(smem + up));
+                const float2 ed = sub_f32x2(P, *reinterpret_cast<const unsigned long long*>(smem + dn));
+                au = fabsf(eu.x) < t;
+                ad = fabsf(ed.x) < t;
+                const float du = fmaxf(fabsf(eu.x), fabsf(eu.y));
+                const float dd = fmaxf(fabsf(ed.x), fabsf(ed.y));
                 insert2<KK>(best, fminf(du, dd), fmaxf(du, dd));
-                up += au ? 1 : 0;
-                dn -= ad ? 1 : 0;
-                if (!au && !ad) inblk = false;
+                up += au ? (int)sizeof(float2) : 0;
+                dn -= ad ? (int)sizeof(float2) : 0;
             }
+            inblk = au || ad;  // a closed side stays closed: the threshold only shrinks
         }
         const bool aborted = steps > step_bound;
         group_sync(group);
 
         // ---- marginal counts and the digamma sum, evenly split over the group
-        const bool dbg = A.dbg_eps && r == 0 && v == A.v_begin;
-        double acc = 0.0;
-        const int top = pow2_floor(M);
-        for (int pos = gt; pos < nb * kBlk; pos += GT) {
-            const int b = pos / kBlk, p = pos - b * kBlk;
-            if (p >= min(kBlk, M - b * kBlk)) continue;
+        long long acc = 0;  // fixed point
+        for (int pos = gt; pos < M; pos += GT) {
+            const int b = pos >> lw;
             const float e = eps_s[pos];
-            const float2 me = blk[1 + b * kBlkStride + p];
+            float2 me = blk[1 + b + pos];
+            if (constant) me = make_float2(me.y, me.x);
             int cx, cy;
             if (A.variant == 2) {  // non-strict counts within the k-NN set's marginal extents
                 float ex, ey;
-                block_extents(blk, bx, nb, b, me.y, me.x, e, ex, ey);
+                block_extents(blk, bx, M, nb, lw, b, me.y, me.x, e, ex, ey);
                 count_le_pair(xsg, ys, M, top, me.y, ex, me.x, ey, cx, cy);
-                acc += A.psi[cx - 1] + A.psi[cy - 1];  // the member itself excluded
+                --cx;  // the member itself excluded
+                --cy;
+                acc += A.psi_fix[cx] + A.psi_fix[cy];
+                if (dbg) {
+                    const int mi = perm[A.dbg_ny[pos]];
+                    A.dbg_eps[mi] = ex;
+                    if (A.dbg_ey) A.dbg_ey[mi] = ey;
+                }
             } else {
                 const int self = e > 0.0f ? 1 : 0;
-                count_within_pair(xsg, ys, M, top, me.y, me.x, e, cx, cy);
+                if (x_shared) count_within_pair(xsh, ys, M, top, me.y, me.x, e, cx, cy);
+                else count_within_pair(xsg, ys, M, top, me.y, me.x, e, cx, cy);
                 cx -= self;
                 cy -= self;
-                acc += A.psi[cx + 1] + A.psi[cy + 1];
+                acc += A.psi_fix[cx + 1] + A.psi_fix[cy + 1];
+                if (dbg) {
+                    const int mi = perm[A.dbg_ny[pos]];
+                    A.dbg_eps[mi] = e;
+                    if (A.dbg_ey) A.dbg_ey[mi] = e;
+                }
             }
-            if (dbg) A.dbg_nx[pos] = __float_as_int(e);  // eps by block position (scratch)
+            if (dbg) A.dbg_nx[pos] = cx | (cy << 16);  // counts by block position (scratch)
         }
         if (dbg) {
-            // member ids: each block's sort again (deterministic) gives its positions' x-ranks.
-            // Pass 1 moves eps from the position-indexed scratch (dbg_nx) to dbg_eps[member];
-            // after every read of the scratch, pass 2 writes the counts over it.
+            // the counts in member order: every thread first moves its positions' scratch (x-rank,
+            // counts) to shared memory that is no longer read, then all write the results over it
             group_sync(group);
-            for (int bq = gw; bq < nb; bq += kGroupWarps) {
-                float key[kBlkRegs];
-                int val[kBlkRegs];
-                block_keys(A, perm, bq, v, key, val);
-                warp_sort_block(key, val);
-#pragma unroll
-                for (int r2 = 0; r2 < kBlkRegs; ++r2)
-                    if (val[r2] < M)
-                        A.dbg_eps[perm[val[r2]]] = __int_as_float(A.dbg_nx[bq * kBlk + r2 * 32 + lane]);
-            }
+            for (int pos = gt; pos < M; pos += GT)
+                blk[1 + pos] = make_float2(__int_as_float(A.dbg_ny[pos]), __int_as_float(A.dbg_nx[pos]));
             group_sync(group);
-            for (int bq = gw; bq < nb; bq += kGroupWarps) {
-                float key[kBlkRegs];
-                int val[kBlkRegs];
-                block_keys(A, perm, bq, v, key, val);
-                warp_sort_block(key, val);
-#pragma unroll
-                for (int r2 = 0; r2 < kBlkRegs; ++r2) {
-                    if (val[r2] >= M) continue;
-                    const int mi = perm[val[r2]];
-                    const float e = A.dbg_eps[mi];
-                    const float2 me = blk[1 + bq * kBlkStride + r2 * 32 + lane];
-                    if (A.variant == 2) {  // extents, then non-strict counts (self excluded)
-                        float ex, ey;
-                        block_extents(blk, bx, nb, bq, me.y, me.x, e, ex, ey);
-                        A.dbg_eps[mi] = ex;
-                        if (A.dbg_ey) A.dbg_ey[mi] = ey;
-                        A.dbg_nx[mi] = count_le([&](int j) { return xsg[j]; }, M, me.y, ex) - 1;
-                        A.dbg_ny[mi] = count_le([&](int j) { return ys[j]; }, M, me.x, ey) - 1;
-                        continue;
-                    }
-                    const int self = e > 0.0f ? 1 : 0;
-                    if (A.dbg_ey) A.dbg_ey[mi] = e;
-                    A.dbg_nx[mi] = count_within(xsg, M, me.y, e) - self;
-                    A.dbg_ny[mi] = count_within(ys, M, me.x, e) - self;
-                }
+            for (int pos = gt; pos < M; pos += GT) {
+                const float2 c = blk[1 + pos];
+                const int mi = perm[__float_as_int(c.x)], n = __float_as_int(c.y);
+                A.dbg_nx[mi] = n & 0xffff;
+                A.dbg_ny[mi] = n >> 16;
             }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
-        evals_total += __reduce_add_sync(FULL, my_evals);
-        if (lane == 0) ctl->part[gw] = aborted ? __longlong_as_double(0x7ff8000000000000ll) : acc;
+        evals_total += __reduce_add_sync(FULL, my_evals / (unsigned)sizeof(float2));
+        if (lane == 0) ctl->part[gw] = aborted ? LLONG_MIN : acc;
         group_sync(group);
         if (gt == 0) {
-            double tot = 0.0;
+            long long sum = 0;
+            bool gave_up = false;
 #pragma unroll
-            for (int w = 0; w < kGroupWarps; ++w) tot += ctl->part[w];
-            const double mi = psi_k - (A.variant == 2 ? 1.0 / A.k : 0.0) + psi_M - tot / (double)M;
+            for (int w = 0; w < kGroupWarps; ++w) {
+                sum += ctl->part[w];
+                gave_up = gave_up || ctl->part[w] == LLONG_MIN;
+            }
+            const double tot = (double)sum * (1.0 / (double)(1ll << kPsiFixBits));
+            double mi = psi_k - (A.variant == 2 ? 1.0 / A.k : 0.0) + psi_M - tot / (double)M;
+            if (gave_up) mi = __longlong_as_double(0x7ff8000000000000ll);
             A.out[A.paired ? (v - A.v_begin) : (int64_t)r * A.out_stride + (v - A.v_begin)] = (float)mi;
             if (dbg && A.dbg_mi) *A.dbg_mi = mi;
         }
@@ -1202,23 +1355,24 @@ static cudaError_t launch_ksg_k(ndf_ctx* ctx, KsgArgs A, bool prune) {
     const int M = A.M;
     if (prune && ctx->ksg_algorithm == NDF_KSG_LANES && (A.variant == 1 || A.variant == 2)) {
         // two-warp groups per pair; as many groups per CTA as fit in shared memory
-        const size_t per_group = lane_group_bytes(M);
-        int gpc = (int)((227 * 1024) / per_group);
-        if (gpc > kMaxGroupsPerCta) gpc = kMaxGroupsPerCta;
+        const int lw = lane_block_log2(M);
+        const size_t per_group = (size_t)LaneSmem(M, lw).total;
+        const size_t shared_x = A.R == 1 ? sizeof(float) * (size_t)M : 0;
+        const int64_t pairs = A.paired ? (A.v_end - A.v_begin) : (int64_t)A.R * (A.v_end - A.v_begin);
+        int gpc = (int)((227 * 1024 - shared_x) / per_group);
+        if (gpc > kLaneMaxGroups) gpc = kLaneMaxGroups;
+        // fewer pairs than the chip's groups: one CTA per SM, with as few groups as that needs
+        const int64_t need = (pairs + ctx->sm_count - 1) / ctx->sm_count;
+        if (gpc > need) gpc = (int)need;
         if (gpc >= 1) {
-            const size_t smem = (size_t)gpc * per_group;
+            const size_t smem = (size_t)gpc * per_group + shared_x;
             const int threads = 32 * kGroupWarps * gpc;
-            cudaError_t e = ctx->ksg_work.reserve(sizeof(unsigned long long));
-            if (e == cudaSuccess)
-                e = cudaMemsetAsync(ctx->ksg_work.ptr, 0, sizeof(unsigned long long), ctx->stream);
-            if (e != cudaSuccess) return e;
             auto kern = ksg_lane_kernel<K1>;
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            const int64_t pairs = A.paired ? (A.v_end - A.v_begin) : (int64_t)A.R * (A.v_end - A.v_begin);
             int64_t grid = (int64_t)ctx->sm_count;
             if (grid * gpc > pairs) grid = (pairs + gpc - 1) / gpc;
-            kern<<<(unsigned)grid, threads, smem, ctx->stream>>>(A, ctx->ksg_work.as<unsigned long long>(),
+            kern<<<(unsigned)grid, threads, smem, ctx->stream>>>(A, ctx->ksg_work.as<unsigned long long>(), lw,
                                                                  ctx->ksg_switch_min, ctx->ksg_every);
             ctx->launches++;
             return cudaGetLastError();
@@ -1232,12 +1386,8 @@ static cudaError_t launch_ksg_k(ndf_ctx* ctx, KsgArgs A, bool prune) {
         if (gpc >= 1) {
             const size_t smem = (size_t)gpc * per_group;
             const int threads = 32 * kGroupWarps * gpc;
-            cudaError_t e = ctx->ksg_work.reserve(sizeof(unsigned long long));
-            if (e == cudaSuccess)
-                e = cudaMemsetAsync(ctx->ksg_work.ptr, 0, sizeof(unsigned long long), ctx->stream);
-            if (e != cudaSuccess) return e;
             auto kern = ksg_block_kernel<K1>;
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             const int64_t pairs = A.paired ? (A.v_end - A.v_begin) : (int64_t)A.R * (A.v_end - A.v_begin);
             int64_t grid = (int64_t)ctx->sm_count;
@@ -1255,12 +1405,8 @@ static cudaError_t launch_ksg_k(ndf_ctx* ctx, KsgArgs A, bool prune) {
         if (gpc < 1) gpc = 1;
         const size_t smem = (size_t)gpc * per_group;
         const int threads = 32 * kGroupWarps * gpc;
-        cudaError_t e = ctx->ksg_work.reserve(sizeof(unsigned long long));
-        if (e == cudaSuccess)
-            e = cudaMemsetAsync(ctx->ksg_work.ptr, 0, sizeof(unsigned long long), ctx->stream);
-        if (e != cudaSuccess) return e;
         auto kern = ksg_pruned_kernel<K1>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
@@ -1300,10 +1446,24 @@ cudaError_t launch_ksg(ndf_ctx* ctx, const Field& rf, const Field& qf, const int
     cudaError_t e = ctx->stage_x.reserve(sizeof(float) * (size_t)M * (size_t)R);
     if (e == cudaSuccess) e = ctx->stage_perm.reserve(sizeof(int) * (size_t)M * (size_t)R);
     if (e != cudaSuccess) return e;
-    ksg_stage_kernel<<<R, 1024, 0, ctx->stream>>>(rf.data, M, rf.N, d_refs, ref0,
-                                                   ctx->stage_x.as<float>(),
-                                                   ctx->stage_perm.as<int>(),
-                                                   ctx->flag.as<unsigned>() + 1);
+    e = ctx->ksg_work.reserve(sizeof(unsigned long long));
+    if (e != cudaSuccess) return e;
+    // a warp per reference where there are many of them, or few members (a lone warp needs about
+    // 0.25 us per register of its lanes)
+    auto stage_warps = [&](auto kern) {
+        const int warps = R < 4 ? R : 4;
+        kern<<<(unsigned)((R + warps - 1) / warps), 32 * warps, 0, ctx->stream>>>(
+            rf.data, M, rf.N, d_refs, ref0, R, ctx->stage_x.as<float>(), ctx->stage_perm.as<int>(),
+            ctx->flag.as<unsigned>() + 1, ctx->ksg_work.as<unsigned long long>());
+    };
+    if (M <= 128) stage_warps(ksg_stage_warp_kernel<4>);
+    else if (M <= 256) stage_warps(ksg_stage_warp_kernel<8>);
+    else if (M <= 512 && R >= 32) stage_warps(ksg_stage_warp_kernel<16>);
+    else if (M <= 1024 && R >= 32) stage_warps(ksg_stage_warp_kernel<32>);
+    else
+        ksg_stage_kernel<<<R, 1024, 0, ctx->stream>>>(rf.data, M, rf.N, d_refs, ref0, ctx->stage_x.as<float>(),
+                                                       ctx->stage_perm.as<int>(), ctx->flag.as<unsigned>() + 1,
+                                                       ctx->ksg_work.as<unsigned long long>());
     ctx->launches++;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     KsgArgs A;
@@ -1320,6 +1480,7 @@ cudaError_t launch_ksg(ndf_ctx* ctx, const Field& rf, const Field& qf, const int
     A.xs_all = ctx->stage_x.as<float>();
     A.perm_all = ctx->stage_perm.as<int>();
     A.psi = ctx->psi.as<double>();
+    A.psi_fix = reinterpret_cast<const long long*>(A.psi + ctx->psi_n);
     A.out = out;
     A.out_stride = out_stride;
     A.dbg_mi = dbg_mi;

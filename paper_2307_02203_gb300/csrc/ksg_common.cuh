@@ -40,43 +40,59 @@ __device__ __forceinline__ int count_within(const float* a, int n, float c, floa
     return hi > lo ? hi - lo : 0;
 }
 
+// Binary searches of several bounds at once over ascending arrays of n values, branchless and
+// without range checks: pred(p) is true up to the bound and false from it on.  A first probe at
+// top - 1 (top = the largest power of two <= n) chooses the window of top - 1 values that holds
+// the bound (the first ones, or the last ones: everything before n - (top - 1) <= top is true
+// then); steps top / 2, .., 1 stay inside it.  One load, one subtract, one compare and one add
+// per bound and step; the bounds' dependent load chains overlap.
+template <int C, class Pred>
+__device__ __forceinline__ void partition_points(int n, int top, int (&pos)[C], Pred&& pred) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) pos[c] = pred(c, top - 1) ? n - (top - 1) : 0;
+#pragma unroll
+    for (int s = 11; s >= 0; --s) {  // n <= 8191
+        const int step = 1 << s;
+        if (step < top) {
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+                if (pred(c, pos[c] + step - 1)) pos[c] += step;
+        }
+    }
+}
+
+// pos[c] = #{p : a[p] < y[c]} in the ascending a[0..n)
+template <int C>
+__device__ __forceinline__ void lower_bounds(const float* a, int n, int top, const float (&y)[C], int (&pos)[C]) {
+    partition_points<C>(n, top, pos, [&](int c, int p) { return a[p] < y[c]; });
+}
+
 // count_within for two arrays at once: na = #{p : |fl(a[p] - c)| < e} in the
-// ascending a[0..n), nb = the same for (b, d).  The four bounds are found by
-// interleaved branchless binary searches over powers of two (top = the largest power
-// of two <= n): each step moves a bound by `step` while the predicate is still false
-// there, so the four dependent load chains overlap.  The predicates are those of
+// ascending a[0..n), nb = the same for (b, d).  The predicates are those of
 // count_within and monotone in p, so the counts are identical.
 __device__ __forceinline__ void count_within_pair(const float* __restrict__ a, const float* __restrict__ b,
                                                   int n, int top, float c, float d, float e, int& na,
                                                   int& nb) {
-    int la = 0, ha = 0, lb = 0, hb = 0;
-    for (int step = top; step > 0; step >>= 1) {
-        const int i1 = la + step, i2 = ha + step, i3 = lb + step, i4 = hb + step;
-        if (i1 <= n && !((c - a[i1 - 1]) < e)) la = i1;   // first p with fl(c - a[p]) < e
-        if (i2 <= n && !((a[i2 - 1] - c) >= e)) ha = i2;  // first p with fl(a[p] - c) >= e
-        if (i3 <= n && !((d - b[i3 - 1]) < e)) lb = i3;
-        if (i4 <= n && !((b[i4 - 1] - d) >= e)) hb = i4;
-    }
-    na = ha > la ? ha - la : 0;
-    nb = hb > lb ? hb - lb : 0;
+    int q[4];
+    partition_points<4>(n, top, q, [&](int i, int p) {
+        return i == 0 ? !((c - a[p]) < e) : i == 1 ? !((a[p] - c) >= e) : i == 2 ? !((d - b[p]) < e) : !((b[p] - d) >= e);
+    });
+    na = q[1] > q[0] ? q[1] - q[0] : 0;
+    nb = q[3] > q[2] ? q[3] - q[2] : 0;
 }
 
 // The non-strict counts of KSG algorithm 2 for two arrays at once, by the same
-// interleaved searches: na = #{p : |fl(a[p] - c)| <= ea}, nb = #{p : |fl(b[p] - d)| <= eb}
+// searches: na = #{p : |fl(a[p] - c)| <= ea}, nb = #{p : |fl(b[p] - d)| <= eb}
 // (the predicates of count_le).
 __device__ __forceinline__ void count_le_pair(const float* __restrict__ a, const float* __restrict__ b, int n,
                                               int top, float c, float ea, float d, float eb, int& na,
                                               int& nb) {
-    int la = 0, ha = 0, lb = 0, hb = 0;
-    for (int step = top; step > 0; step >>= 1) {
-        const int i1 = la + step, i2 = ha + step, i3 = lb + step, i4 = hb + step;
-        if (i1 <= n && !((c - a[i1 - 1]) <= ea)) la = i1;  // first p with fl(c - a[p]) <= ea
-        if (i2 <= n && !((a[i2 - 1] - c) > ea)) ha = i2;   // first p with fl(a[p] - c) > ea
-        if (i3 <= n && !((d - b[i3 - 1]) <= eb)) lb = i3;
-        if (i4 <= n && !((b[i4 - 1] - d) > eb)) hb = i4;
-    }
-    na = ha > la ? ha - la : 0;
-    nb = hb > lb ? hb - lb : 0;
+    int q[4];
+    partition_points<4>(n, top, q, [&](int i, int p) {
+        return i == 0 ? !((c - a[p]) <= ea) : i == 1 ? !((a[p] - c) > ea) : i == 2 ? !((d - b[p]) <= eb) : !((b[p] - d) > eb);
+    });
+    na = q[1] > q[0] ? q[1] - q[0] : 0;
+    nb = q[3] > q[2] ? q[3] - q[2] : 0;
 }
 
 // the largest power of two <= n (n >= 1)

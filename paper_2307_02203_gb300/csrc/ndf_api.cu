@@ -198,12 +198,18 @@ double digamma_int_host(int64_t n) {
 ndf_status ensure_psi_table(ndf_ctx* ctx, int64_t n_max) {
     if (ctx->psi_n > n_max) return NDF_OK;
     int64_t n = n_max + 1;
+    // n doubles, then the same values in fixed point
     std::vector<double> h((size_t)n, 0.0);
-    for (int64_t i = 1; i < n; ++i) h[(size_t)i] = digamma_int_host(i);
-    cudaError_t e = ctx->psi.reserve(sizeof(double) * (size_t)n);
+    std::vector<int64_t> fix((size_t)n, 0);
+    for (int64_t i = 1; i < n; ++i) {
+        h[(size_t)i] = digamma_int_host(i);
+        fix[(size_t)i] = (int64_t)llrint(ldexp(h[(size_t)i], kPsiFixBits));
+    }
+    const size_t bytes = sizeof(double) * (size_t)n;
+    cudaError_t e = ctx->psi.reserve(2 * bytes);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->psi.ptr, h.data(), bytes, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ctx->psi.ptr, h.data(), sizeof(double) * (size_t)n,
-                            cudaMemcpyHostToDevice, ctx->stream);
+        e = cudaMemcpyAsync(ctx->psi.as<double>() + n, fix.data(), bytes, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "digamma table upload");
     ctx->psi_n = n;

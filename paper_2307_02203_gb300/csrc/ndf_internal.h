@@ -109,7 +109,10 @@ ndf_status resolve_out(ndf_ctx* ctx, void* out, size_t bytes, void** dev_out, bo
 ndf_status check_device_status(ndf_ctx* ctx);
 ndf_status finish_out(ndf_ctx* ctx, void* out, const void* dev_out, size_t bytes, bool is_host);
 
-// Digamma psi(n) for n = 0..n_max (entry 0 unused), FP64, on the device.
+// Digamma psi(n) for n = 0..n_max (entry 0 unused), FP64, on the device (ctx->psi, psi_n
+// entries), followed by the same values in fixed point, psi 2^kPsiFixBits rounded: sums of up to
+// 2 x 4096 of them stay below 2^63 and do not depend on their order.
+constexpr int kPsiFixBits = 45;
 ndf_status ensure_psi_table(ndf_ctx* ctx, int64_t n_max);
 double digamma_int_host(int64_t n);
 
