@@ -40,13 +40,13 @@ __device__ __forceinline__ void vertex_pos(int64_t v, int64_t X, int64_t Y, int6
     p[2] = axis_pos(z, Z);
 }
 
-static uint64_t host_mix(uint64_t z) {
+__host__ __device__ static inline uint64_t host_mix(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
     z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
     return z ^ (z >> 31);
 }
 
-static uint64_t host_rand(uint64_t key, uint64_t i) {
+__host__ __device__ static inline uint64_t host_rand(uint64_t key, uint64_t i) {
     return host_mix(key + (i + 1) * 0x9e3779b97f4a7c15ULL);
 }
 
@@ -95,6 +95,25 @@ __device__ __forceinline__ float lerp_rn(float a, float b, float t) {
     return __fadd_rn(__fmul_rn(a, __fsub_rn(1.0f, t)), __fmul_rn(b, t));
 }
 
+// positions of pairs c0 .. c0 + n - 1: six draws each on a 24-bit uniform grid on [-1, 1)
+// (k 2^-23 - 1 with k < 2^24: every step exact in FP32).  Drawn on the device: the host loop and
+// its uploads took 1.5 ms per 100,000 pairs.
+__global__ void sample_positions_kernel(uint64_t key, int64_t c0, int64_t n, float* __restrict__ pref,
+                                        float* __restrict__ pq) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+        const float v = (float)(int)(host_rand(key, (uint64_t)((c0 + i) * 6 + d)) >> 40) * 0x1.0p-23f - 1.0f;
+        if (d < 3) pref[3 * i + d] = v;
+        else pq[3 * i + d - 3] = v;
+    }
+}
+
+// VEC (N and the base 16-byte aligned): the two x-neighbours of a row come from one aligned
+// 16-byte load (three positions in four) or that and a 4-byte one, not two 4-byte ones: every
+// lane's row is another sector, so the kernel is bound by the requests, not by the bytes.
+template <bool VEC>
 __global__ void interp_columns_kernel(const float* __restrict__ field, int64_t M, int64_t X,
                                       int64_t Y, int64_t Z, const float* __restrict__ pos,
                                       int64_t n, float* __restrict__ out) {
@@ -110,12 +129,25 @@ __global__ void interp_columns_kernel(const float* __restrict__ field, int64_t M
     const int64_t o010 = (z0 * Y + y1) * X + x0, o110 = (z0 * Y + y1) * X + x1;
     const int64_t o001 = (z1 * Y + y0) * X + x0, o101 = (z1 * Y + y0) * X + x1;
     const int64_t o011 = (z1 * Y + y1) * X + x0, o111 = (z1 * Y + y1) * X + x1;
+    const bool two = x1 > x0;
+    // (value at x0, value at x1) of a row: o its index at x0
+    auto pair = [&](const float* f, int64_t o, int64_t o1) {
+        if (!VEC) return make_float2(__ldg(f + o), __ldg(f + o1));
+        const int r = (int)(o & 3);
+        const float4 v = __ldg(reinterpret_cast<const float4*>(f + (o - r)));
+        float2 c;
+        c.x = r < 2 ? (r == 0 ? v.x : v.y) : (r == 2 ? v.z : v.w);
+        c.y = r < 2 ? (r == 0 ? v.y : v.z) : v.w;
+        if (r == 3 && two) c.y = __ldg(f + o1);
+        if (!two) c.y = c.x;
+        return c;
+    };
     for (int64_t m = blockIdx.y; m < M; m += gridDim.y) {
         const float* f = field + m * N;
-        const float c00 = lerp_rn(__ldg(f + o000), __ldg(f + o100), wx);
-        const float c10 = lerp_rn(__ldg(f + o010), __ldg(f + o110), wx);
-        const float c01 = lerp_rn(__ldg(f + o001), __ldg(f + o101), wx);
-        const float c11 = lerp_rn(__ldg(f + o011), __ldg(f + o111), wx);
+        const float2 a = pair(f, o000, o100), b = pair(f, o010, o110);
+        const float2 c = pair(f, o001, o101), d = pair(f, o011, o111);
+        const float c00 = lerp_rn(a.x, a.y, wx), c10 = lerp_rn(b.x, b.y, wx);
+        const float c01 = lerp_rn(c.x, c.y, wx), c11 = lerp_rn(d.x, d.y, wx);
         out[m * n + i] = lerp_rn(lerp_rn(c00, c10, wy), lerp_rn(c01, c11, wy), wz);
     }
 }
@@ -163,30 +195,21 @@ cudaError_t sample_triples_dev(ndf_ctx* ctx, const Field& rf, const Field& qf, i
     cudaError_t e = sc.reserve(M, chunk);
     if (e != cudaSuccess) return e;
     const uint64_t key = host_mix(seed ^ 0x434f4e54504f5353ULL);
-    std::vector<float> hp((size_t)chunk * 6);
     int* d_flag = ctx->flag.as<int>();
     for (int64_t c0 = 0; c0 < n && e == cudaSuccess; c0 += chunk) {
         const int64_t nc = std::min(chunk, n - c0);
-        // 24-bit uniform grid on [-1, 1): exact in FP32
-        for (int64_t i = 0; i < nc * 6; ++i)
-            hp[(size_t)i] = (float)((double)(host_rand(key, (uint64_t)(c0 * 6 + i)) >> 40) *
-                                        (2.0 / 16777216.0) - 1.0);
-        std::vector<float> hr((size_t)nc * 3), hq((size_t)nc * 3);
-        for (int64_t i = 0; i < nc; ++i)
-            for (int d = 0; d < 3; ++d) {
-                hr[(size_t)(3 * i + d)] = hp[(size_t)(6 * i + d)];
-                hq[(size_t)(3 * i + d)] = hp[(size_t)(6 * i + 3 + d)];
-            }
-        e = cudaMemcpyAsync(pref + 3 * c0, hr.data(), (size_t)nc * 12, cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(pq + 3 * c0, hq.data(), (size_t)nc * 12, cudaMemcpyHostToDevice, ctx->stream);
-        if (e != cudaSuccess) break;
+        sample_positions_kernel<<<(unsigned)((nc + 127) / 128), 128, 0, ctx->stream>>>(key, c0, nc, pref + 3 * c0,
+                                                                                      pq + 3 * c0);
         const dim3 grid((unsigned)((nc + 127) / 128), (unsigned)std::min<int64_t>(M, 64));
-        interp_columns_kernel<<<grid, 128, 0, ctx->stream>>>(rf.data, M, rf.X, rf.Y, rf.Z,
-                                                             pref + 3 * c0, nc, sc.ca);
-        interp_columns_kernel<<<grid, 128, 0, ctx->stream>>>(qf.data, M, qf.X, qf.Y, qf.Z,
-                                                             pq + 3 * c0, nc, sc.cb);
-        ctx->launches += 2;
+        auto interp = [&](const Field& f, const float* pos, float* out) {
+            if ((f.N & 3) == 0 && ((uintptr_t)f.data & 15) == 0)
+                interp_columns_kernel<true><<<grid, 128, 0, ctx->stream>>>(f.data, M, f.X, f.Y, f.Z, pos, nc, out);
+            else
+                interp_columns_kernel<false><<<grid, 128, 0, ctx->stream>>>(f.data, M, f.X, f.Y, f.Z, pos, nc, out);
+        };
+        interp(rf, pref + 3 * c0, sc.ca);
+        interp(qf, pq + 3 * c0, sc.cb);
+        ctx->launches += 3;
         Field fa, fb;
         fa.live = fb.live = true;
         fa.M = fb.M = M;
@@ -215,10 +238,8 @@ cudaError_t sample_triples_dev(ndf_ctx* ctx, const Field& rf, const Field& qf, i
                 e = launch_ksg(ctx, fa, fb, nullptr, 0, (int)nc, k, 0, nc, target + c0, 0, true, 1, 1,
                                nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr, true);
         }
-        // the host position buffers and the column blocks are reused by the next chunk
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     }
-    return e;
+    return e == cudaSuccess ? cudaStreamSynchronize(ctx->stream) : e;
 }
 
 // Sum of the training targets (FP64, one atomic per block), for the MI network's
