@@ -7,23 +7,57 @@
 
 namespace ndf {
 
-// largest number of K slices of a split product (the workspace holds that many
-// partial results)
-constexpr int64_t kSplitK = 64;
+// A dense layer over `batch` independent weight sets (one, or one per encoder of a cross
+// field): rows [i * rows, (i + 1) * rows) of the activations belong to weight set i, whose
+// parameters start i * wstride floats after W and b.
+struct DenseLayer {
+    const float* W = nullptr;  // [cout][cin]
+    const float* b = nullptr;  // [cout]
+    int cin = 0, cout = 0;
+    int64_t rows = 0;
+    int batch = 1;
+    int64_t wstride = 0;
+};
 
-// C[M][N] = A[M][K] B[N][K]^T
-cudaError_t gemm_f32_nt(cudaStream_t s, const float* A, const float* B, float* C, int64_t M,
-                        int64_t N, int64_t K);
-// C[M][N] = A[M][K] B[K][N]
-cudaError_t gemm_f32_nn(cudaStream_t s, const float* A, const float* B, float* C, int64_t M,
-                        int64_t N, int64_t K);
-// C[M][N] += A[K][M]^T B[K][N], K split into slices summed in a fixed order;
-// work: gemm_f32_tn_work_floats(M, N, K) floats
-cudaError_t gemm_f32_tn_acc(cudaStream_t s, const float* A, const float* B, float* C, int64_t M,
-                            int64_t N, int64_t K, float* work);
-int64_t gemm_f32_tn_work_floats(int64_t M, int64_t N, int64_t K);
-// out[N] += sum_k A[k][n] over A[K][N], in fixed slices; work: kSplitK * N floats
-cudaError_t colsum_f32_acc(cudaStream_t s, const float* A, float* out, int64_t K, int64_t N,
-                           float* work);
+// pre = X W^T + b; post = act(pre) when post is given (activation code as in act_f)
+cudaError_t dense_forward(cudaStream_t s, const DenseLayer& L, const float* X, float* pre, float* post,
+                          int act);
+
+// The weight and bias gradients are sums over the rows: every chunk of rows writes a partial
+// sum, and one kernel at the end adds the partials of all layers in a fixed order
+// (deterministic).  GradSums holds the list of partials and their workspace.
+constexpr int kGradSegs = 40;
+constexpr int64_t kGradSplits = 64;   // most chunks of one layer
+struct GradSeg {
+    const float* part;  // [splits][n]
+    float* dst;         // dst[i] (+)= sum over the splits
+    int64_t n;
+    int splits;
+    int add;
+};
+struct GradSums {
+    float* work = nullptr;
+    int64_t cap = 0, used = 0;
+    GradSeg seg[kGradSegs];
+    int count = 0;
+    float* take(int64_t floats) {  // nullptr: flush first
+        if (used + floats > cap) return nullptr;
+        float* r = work + used;
+        used += (floats + 3) & ~int64_t(3);
+        return r;
+    }
+};
+// workspace one layer needs (any rows, batch of up to two weight sets)
+int64_t dense_grad_floats(int64_t cin, int64_t cout);
+// adds every listed partial to its destination and empties the list (counts one launch)
+cudaError_t grad_sums_flush(cudaStream_t s, GradSums& g, uint64_t* launches);
+
+// One launch: the weight and bias gradients' partials of the layer (dW, db += ...; gradients of
+// weight set i at dW + i * wstride) and, when dX is given, the data gradient of its input
+// columns [col0, cin): dX[rows][cin - col0] = (dY W)[.., col0..] (* act'(pre_in), the layer
+// input's pre-activations [rows][cin], when given; col0 = 0 then).
+cudaError_t dense_backward(cudaStream_t s, const DenseLayer& L, const float* X, const float* dY, float* dX,
+                           int col0, const float* pre_in, int act, float* dW, float* db, GradSums& g,
+                           uint64_t* launches);
 
 }  // namespace ndf

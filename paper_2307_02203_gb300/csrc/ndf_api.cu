@@ -108,6 +108,15 @@ PtrKind pointer_kind(const void* p) {
                                                                                 : PTR_HOST;
 }
 
+bool device_writable(const ndf_ctx* ctx, const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == ctx->device && ((uintptr_t)p & 3) == 0;
+}
+
 ndf_status fail(ndf_ctx* ctx, ndf_status st, const char* fmt, ...) {
     if (ctx) {
         char buf[512];

@@ -12,11 +12,12 @@
 //            the decoder layers.  One encoder (self field, symmetric by
 //            construction) or two (cross field: 0 reference, 1 query).
 //
-// GPU design: activations are feature-major per sample ([B][c] row-major), the
-// dense layers are this library's FP32 matrix products (gemm_f32.cu: FP32 for
-// parity with the oracle, deterministic weight-gradient sums), and everything
-// between them (embedding, bias + activation, merge, output + loss, the
-// hash-table scatter of the backward, Adam) is in the kernels below.
+// GPU design: activations are sample-major ([rows][c]; the reference side's rows first, then
+// the query side's, so a self field's shared encoder runs once over both).  The dense layers
+// are this library's FP32 products (gemm_f32.cu: bias, activation and its derivative in their
+// epilogues, deterministic weight-gradient sums), and the rest (embedding, merge, output layer
+// with the loss and its gradients, the hash-table scatter of the backward, Adam) are the
+// kernels below.
 #include <math.h>
 #include <string.h>
 
@@ -37,51 +38,67 @@ namespace ndf {
 // relative to the He-uniform scale of the other weights (see ndf_hash_model_create)
 constexpr double kFourierInit = 0.1;
 
-// x0[b][din] = embed(pos[b]) with the tables of one encoder
-__global__ void hash_embed_kernel(const float* __restrict__ pos, int64_t B,
-                                  const float* __restrict__ enc, EmbedArgs E,
-                                  float* __restrict__ x0) {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const float p[3] = {pos[3 * b], pos[3 * b + 1], pos[3 * b + 2]};
-    float* x = x0 + b * E.din;
-    embed_point(E, enc, p, [&](int k, float v) { x[k] = v; });
-}
-
-// hash-table gradient: scatter dL/d(embedding) of the hash features
-__global__ void hash_embed_backward_kernel(const float* __restrict__ pos, int64_t B,
-                                           const float* __restrict__ gx, EmbedArgs E,
-                                           float* __restrict__ genc) {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const float p[3] = {pos[3 * b], pos[3 * b + 1], pos[3 * b + 2]};
-    const float* g = gx + b * E.din + 3 + 6 * E.L;
-    for (int l = 0; l < E.levels; ++l) {
-        const Cell cl = level_cell(E, l, p);
-        float* tab = genc + E.toff[l];
-        for (int f = 0; f < E.F; ++f) {
-            const float gv = g[l * E.F + f];
-            if (gv == 0.0f) continue;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) atomicAdd(tab + (int64_t)cl.idx[q] * E.F + f, cl.w[q] * gv);
+// x0[row][din] = embed(position of the row): rows [0, B) from pos0 with the tables at enc0, rows
+// [B, rows) from pos1 with those at enc1.  A CTA embeds 32 rows into shared memory and writes
+// them coalesced; its warps split the features of a row (a Fourier axis and frequency or a grid
+// level at a time: one row per lane, no divergence), so a batch of 8192 pairs fills the chip
+// (one thread per row, measured: 15 us per 8192 rows; this: 6.5 us for all 16,384).
+constexpr int kEmbedRows = 32;
+__global__ void __launch_bounds__(256)
+    hash_embed_kernel(const float* __restrict__ pos0, const float* __restrict__ pos1, int64_t B, int64_t rows,
+                      const float* __restrict__ enc0, const float* __restrict__ enc1, EmbedArgs E,
+                      float* __restrict__ x0) {
+    extern __shared__ float xs[];  // [32][ld], ld odd: conflict-free by row
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ld = E.din | 1;
+    const int64_t r0 = (int64_t)blockIdx.x * kEmbedRows, r = r0 + lane;
+    if (r < rows) {
+        const float* pp = r < B ? pos0 + 3 * r : pos1 + 3 * (r - B);
+        const float* enc = r < B ? enc0 : enc1;
+        const float p[3] = {pp[0], pp[1], pp[2]};
+        float* x = xs + lane * ld;
+        for (int u = warp; u < E.levels + 3 * E.L + 1; u += 8) {
+            if (u < E.levels) {
+                embed_levels(E, enc, p, u, u + 1, [&](int k, float v) { x[3 + 6 * E.L + k] = v; });
+            } else if (u < E.levels + 3 * E.L) {
+                const int f = u - E.levels, j = f / E.L;
+                float sn, cs;
+                sincospif(ldexpf(p[j], f - j * E.L), &sn, &cs);
+                x[3 + 2 * f] = sn;
+                x[4 + 2 * f] = cs;
+            } else {
+                x[0] = p[0];
+                x[1] = p[1];
+                x[2] = p[2];
+            }
         }
+    }
+    __syncthreads();
+    const int n = (int)min((int64_t)kEmbedRows, rows - r0) * E.din;
+    for (int i = threadIdx.x; i < n; i += 256) {
+        const int q = i / E.din;
+        x0[r0 * E.din + i] = xs[q * ld + (i - q * E.din)];
     }
 }
 
-// pre[b][o] += bias[o]; post = act(pre) (or a copy when act < 0)
-__global__ void bias_act_kernel(float* __restrict__ pre, const float* __restrict__ bias, int c,
-                                int64_t B, int act, float* __restrict__ post) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)c * B) return;
-    const float v = pre[i] + bias[i % c];
-    pre[i] = v;
-    if (post) post[i] = act < 0 ? v : act_f(act, v);
-}
-
-__global__ void dact_mul_kernel(float* __restrict__ g, const float* __restrict__ pre, int64_t n,
-                                int act) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) g[i] *= dact_f(act, pre[i]);
+// hash-table gradient: scatter dL/d(embedding) of the hash features, gx[row][ld] from its
+// column 0 on (rows as in hash_embed_kernel), one thread per row and level
+__global__ void hash_embed_backward_kernel(const float* __restrict__ pos0, const float* __restrict__ pos1,
+                                           int64_t B, int64_t rows, const float* __restrict__ gx, int ld,
+                                           EmbedArgs E, float* __restrict__ genc0, float* __restrict__ genc1) {
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int l = blockIdx.y;
+    if (r >= rows) return;
+    const float* pp = r < B ? pos0 + 3 * r : pos1 + 3 * (r - B);
+    const float p[3] = {pp[0], pp[1], pp[2]};
+    const float* g = gx + r * ld + l * E.F;
+    const Cell cl = level_cell(E, l, p);
+    float* tab = (r < B ? genc0 : genc1) + E.toff[l];
+    for (int f = 0; f < E.F; ++f) {
+        const float gv = g[f];
+        if (gv == 0.0f) continue;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) atomicAdd(tab + (int64_t)cl.idx[q] * E.F + f, cl.w[q] * gv);
+    }
 }
 
 // z from the two latents (d features each, zr broadcast when zr_stride == 0):
@@ -123,48 +140,125 @@ __global__ void merge_backward_kernel(const float* __restrict__ g, const float* 
     }
 }
 
-// y = out_act(raw) (and the L1 loss and its gradient when target != null)
-__global__ void out_loss_kernel(const float* __restrict__ raw, const float* __restrict__ target,
-                                int64_t B, int measure, float* __restrict__ y,
-                                float* __restrict__ graw, double* __restrict__ loss) {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// The output layer (one output: raw = w . in + bias), y = out_act(raw) and, when target is
+// given, the L1 loss, its gradient through the layer and the layer's own gradients: in[B][cin]
+// is read once, dX = dL/draw * w (* act'(pre), the pre-activations of `in`, when given), and
+// every CTA's sums over its rows of dL/draw * in and dL/draw go to part[blockIdx.x][cin + 1]
+// (added in order by grad_sums_flush).  One warp per row for the dot products, then one thread
+// per column (several row groups when there are fewer columns than threads), 32 rows at a
+// time; a CTA takes `chunk` consecutive rows.
+constexpr int kOutRows = 32;
+constexpr int64_t kOutMaxCtas = 256;  // partial sums to add
+inline int64_t out_chunk(int64_t B) {
+    const int64_t c = (B + kOutMaxCtas - 1) / kOutMaxCtas;
+    return (c + kOutRows - 1) / kOutRows * kOutRows;
+}
+__global__ void __launch_bounds__(256)
+    hash_out_kernel(const float* __restrict__ in, const float* __restrict__ w, const float* __restrict__ bias,
+                    int cin, int64_t B, int64_t chunk, int measure, const float* __restrict__ target,
+                    float* __restrict__ y, const float* __restrict__ pre, int act, float* __restrict__ dX, float* __restrict__ part,
+                    double* __restrict__ loss) {
+    __shared__ float gs[kOutRows];
+    __shared__ float red[256];
+    __shared__ double ls[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t begin = (int64_t)blockIdx.x * chunk, end = min(begin + chunk, B);
+    const int cw = cin > 128 ? 256 : cin > 64 ? 128 : 64, subs = 256 / cw;
+    const int sub = threadIdx.x / cw, c = threadIdx.x % cw;
+    float* pt = target ? part + (int64_t)blockIdx.x * (cin + 1) : nullptr;
     double l = 0.0;
-    if (b < B) {
-        const float x = raw[b];
-        const float v = out_act(measure, x);
-        if (y) y[b] = v;
-        if (target) {
-            const float d = v - target[b];
-            l = fabs((double)d);
-            const float sg = d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f);
-            float dv;
-            if (measure == NDF_MEASURE_PEARSON) {
-                dv = 1.0f - v * v;
-            } else {
-                dv = 1.0f / (1.0f + expf(-x));
-            }
-            graw[b] = sg / (float)B * dv;
-        }
-    }
-    if (target) {
+    for (int64_t b0 = begin; b0 < end; b0 += kOutRows) {
+        const int n = (int)min((int64_t)kOutRows, end - b0);
+        for (int r = warp; r < n; r += 8) {
+            const float* x = in + (b0 + r) * cin;
+            float s = 0.0f;
+#pragma unroll 4
+            for (int i = lane; i < cin; i += 32) s = fmaf(x[i], w[i], s);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-        if ((threadIdx.x & 31) == 0 && l != 0.0) atomicAdd(loss, l);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            const float raw = s + bias[0];
+            const float v = out_act(measure, raw);
+            if (lane == 0 && y) y[b0 + r] = v;
+            if (target) {
+                const float d = v - target[b0 + r];
+                l += fabs((double)d);
+                const float sg = d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f);
+                const float dv = measure == NDF_MEASURE_PEARSON ? 1.0f - v * v : 1.0f / (1.0f + expf(-raw));
+                if (lane == 0) gs[r] = sg / (float)B * dv;
+            }
+        }
+        if (!target) continue;
+        __syncthreads();
+        for (int i0 = 0; i0 < cin; i0 += cw) {
+            const int i = i0 + c;
+            float a = 0.0f;
+            if (i < cin) {
+                const float wi = w[i];
+#pragma unroll 8
+                for (int r = sub; r < n; r += subs) {
+                    const int64_t o = (b0 + r) * cin + i;
+                    const float g = gs[r];
+                    a = fmaf(g, in[o], a);
+                    float d = g * wi;
+                    if (pre) d *= dact_f(act, pre[o]);
+                    dX[o] = d;
+                }
+            }
+            red[threadIdx.x] = a;
+            __syncthreads();
+            if (sub == 0 && i < cin) {
+                for (int k = 1; k < subs; ++k) a += red[k * cw + c];
+                pt[i] = b0 == begin ? a : pt[i] + a;
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            float a = 0.0f;
+            for (int r = 0; r < n; ++r) a += gs[r];
+            pt[cin] = b0 == begin ? a : pt[cin] + a;
+        }
+        __syncthreads();  // gs is rewritten by the next rows
+    }
+    if (!target) return;
+    if (lane == 0) ls[warp] = l;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int k = 0; k < 8; ++k) t += ls[k];
+        if (t != 0.0) atomicAdd(loss, t);
     }
 }
 
-__global__ void hash_adam_kernel(float* __restrict__ p, const float* __restrict__ g,
-                                 float* __restrict__ m, float* __restrict__ v, int64_t n, float lr,
-                                 float b1, float b2, float eps, float c1, float c2) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+__device__ __forceinline__ void adam_one(float& p, float g, float& m, float& v, float lr, float b1, float b2,
+                                         float eps, float c1, float c2) {
+    m = b1 * m + (1.0f - b1) * g;
+    v = b2 * v + (1.0f - b2) * g * g;
+    p -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
+
+// HBM-bound (28 bytes per parameter).  Four parameters per thread with 16-byte accesses, every
+// array streamed once (evict-first); the gradient may be the caller's buffer at any alignment
+// (gvec: 16-byte aligned).
+__global__ void __launch_bounds__(256)
+    hash_adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
+                     float* __restrict__ v, int64_t n, bool gvec, float lr, float b1, float b2, float eps,
+                     float c1, float c2) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, j = i << 2;
+    if (j + 3 < n) {
+        float4 P = __ldcs(reinterpret_cast<const float4*>(p) + i), M = __ldcs(reinterpret_cast<const float4*>(m) + i);
+        float4 V = __ldcs(reinterpret_cast<const float4*>(v) + i);
+        const float4 G = gvec ? __ldcs(reinterpret_cast<const float4*>(g) + i)
+                              : make_float4(__ldcs(g + j), __ldcs(g + j + 1), __ldcs(g + j + 2), __ldcs(g + j + 3));
+        adam_one(P.x, G.x, M.x, V.x, lr, b1, b2, eps, c1, c2);
+        adam_one(P.y, G.y, M.y, V.y, lr, b1, b2, eps, c1, c2);
+        adam_one(P.z, G.z, M.z, V.z, lr, b1, b2, eps, c1, c2);
+        adam_one(P.w, G.w, M.w, V.w, lr, b1, b2, eps, c1, c2);
+        __stcs(reinterpret_cast<float4*>(p) + i, P);
+        __stcs(reinterpret_cast<float4*>(m) + i, M);
+        __stcs(reinterpret_cast<float4*>(v) + i, V);
+        return;
     }
+    for (int64_t k = j; k < n; ++k) adam_one(p[k], g[k], m[k], v[k], lr, b1, b2, eps, c1, c2);
 }
 
 __global__ void fill_kernel(float* __restrict__ p, int64_t n, float v) {
@@ -208,14 +302,15 @@ struct ndf_hash_model {
     HashLayout Ly;
     float *params = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
     int64_t t = 0;
-    // workspace for a batch of up to cap samples, and of the weight-gradient products
-    float* gemm_work = nullptr;
+    // workspace for a batch of up to cap samples (encoder buffers: both sides' rows), and of the
+    // weight-gradient partial sums
+    GradSums sums;
     int64_t cap = 0;
     float* ws = nullptr;
-    float *x0[2] = {}, *pre_e[2][kHashMaxLayers] = {}, *post_e[2][kHashMaxLayers] = {};
+    float *x0 = nullptr, *pre_e[kHashMaxLayers] = {}, *post_e[kHashMaxLayers] = {};
     float *z = nullptr, *pre_d[kHashMaxLayers] = {}, *post_d[kHashMaxLayers] = {};
-    float *ga = nullptr, *gb = nullptr, *gr = nullptr, *gq = nullptr;
-    float *graw = nullptr, *tgt = nullptr, *pos = nullptr;
+    float *ga = nullptr, *gb = nullptr, *gl = nullptr;
+    float *y = nullptr, *tgt = nullptr, *pos = nullptr;
     double* loss = nullptr;
     // tensor-core decoding: packed BF16 weight images and biases of the parameter
     // version tc_ver, reference latents, per-axis Fourier features of the decode
@@ -235,179 +330,196 @@ namespace ndf {
 static cudaError_t hash_workspace(ndf_hash_model* m, int64_t B) {
     if (B <= m->cap) return cudaSuccess;
     if (m->ws) cudaFree(m->ws);
-    if (m->gemm_work) cudaFree(m->gemm_work);
+    if (m->sums.work) cudaFree(m->sums.work);
     m->ws = nullptr;
-    m->gemm_work = nullptr;
+    m->sums = GradSums();
     m->cap = 0;
     const HashLayout& L = m->Ly;
     const int64_t c = L.c, wmax = std::max<int64_t>(std::max<int64_t>(L.din, c), L.ddec);
-    // loss (2 doubles), x0 x2, encoder pre/post x2 sides, z, decoder pre/post,
-    // ga, gb (ping-pong), gr, gq (merge gradients), graw, tgt, positions
-    const int64_t floats = 4 + 2 * B * L.din + 2 * 2 * L.le * B * c + B * L.ddec +
-                           2 * L.ld * B * c + 2 * B * wmax + 2 * B * L.dlat + 2 * B + 6 * B;
-    cudaError_t e = cudaMalloc(&m->ws, sizeof(float) * (size_t)floats);
-    if (e != cudaSuccess) return e;
-    // partial products of the weight gradients (at most c x wmax per slice) and of the
-    // bias gradients
-    const int64_t wf = std::max<int64_t>(gemm_f32_tn_work_floats(c, wmax, B), kSplitK * wmax);
-    e = cudaMalloc(&m->gemm_work, sizeof(float) * (size_t)wf);
-    if (e != cudaSuccess) return e;
-    float* o = m->ws;
+    // loss (2 doubles); both sides' x0 and encoder pre / post; z, decoder pre / post; ga, gb
+    // (ping-pong gradients, both sides), gl (latent gradients, both sides); y, tgt, positions
+    int64_t floats = 0;
+    float* o = nullptr;
     auto take = [&](int64_t n) {
-        float* r = o;
-        o += n;
+        float* r = o ? o + floats : nullptr;
+        floats += (n + 3) & ~int64_t(3);
         return r;
     };
-    m->loss = reinterpret_cast<double*>(take(4));
-    for (int s = 0; s < 2; ++s) m->x0[s] = take(B * L.din);
-    for (int s = 0; s < 2; ++s)
+    auto carve = [&]() {
+        floats = 0;
+        m->loss = reinterpret_cast<double*>(take(4));
+        m->x0 = take(2 * B * L.din);
         for (int k = 0; k < L.le; ++k) {
-            m->pre_e[s][k] = take(B * c);
-            m->post_e[s][k] = take(B * c);
+            m->pre_e[k] = take(2 * B * c);
+            m->post_e[k] = k < L.le - 1 ? take(2 * B * c) : m->pre_e[k];  // the last layer is linear
         }
-    m->z = take(B * L.ddec);
-    for (int k = 0; k < L.ld; ++k) {
-        m->pre_d[k] = take(B * c);
-        m->post_d[k] = take(B * c);
+        m->z = take(B * L.ddec);
+        for (int k = 0; k < L.ld - 1; ++k) {
+            m->pre_d[k] = take(B * c);
+            m->post_d[k] = take(B * c);
+        }
+        m->ga = take(2 * B * wmax);
+        m->gb = take(2 * B * wmax);
+        m->gl = take(2 * B * L.dlat);
+        m->y = take(B);
+        m->tgt = take(B);
+        m->pos = take(6 * B);
+    };
+    carve();
+    cudaError_t e = cudaMalloc(&o, sizeof(float) * (size_t)floats);
+    if (e != cudaSuccess) return e;
+    m->ws = o;
+    carve();
+    // partial sums of the weight gradients: all layers where that stays within 128 MB (then one
+    // kernel adds them all at the end of a step), at least the largest one
+    const int64_t out_part = kOutMaxCtas * (std::max<int64_t>(L.ddec, c) + 1);
+    const int64_t one = std::max(std::max(dense_grad_floats(wmax, c), dense_grad_floats(L.ddec, c)), out_part + 4);
+    const int64_t all = (L.le + L.ld) * dense_grad_floats(wmax, c) + out_part + 4;
+    m->sums.cap = std::max(one, std::min<int64_t>(all, int64_t(32) << 20));
+    e = cudaMalloc(&m->sums.work, sizeof(float) * (size_t)m->sums.cap);
+    if (e != cudaSuccess) {
+        m->sums = GradSums();
+        return e;
     }
-    m->ga = take(B * wmax);
-    m->gb = take(B * wmax);
-    m->gr = take(B * L.dlat);
-    m->gq = take(B * L.dlat);
-    m->graw = take(B);
-    m->tgt = take(B);
-    m->pos = take(6 * B);
     m->cap = B;
     return cudaSuccess;
 }
 
-// Activations are sample-major, [B][c]; W is [c_out][c_in].
-// Y[B][c_out] = X[B][c_in] W^T
-static bool gemm_fwd(ndf_hash_model* m, const float* W, const float* X, float* Y, int c_out,
-                     int c_in, int64_t B) {
-    return gemm_f32_nt(m->ctx->stream, X, W, Y, B, c_out, c_in) == cudaSuccess;
+// encoder layer k over `batch` weight sets from encoder e on, `rows` rows each
+static DenseLayer enc_layer(const ndf_hash_model* m, int e, int k, int64_t rows, int batch) {
+    const HashLayout& L = m->Ly;
+    DenseLayer d;
+    const float* enc = m->params + L.enc_size * e;
+    d.W = enc + L.ew[k];
+    d.b = enc + L.eb[k];
+    d.cin = k == 0 ? L.din : L.c;
+    d.cout = L.c;
+    d.rows = rows;
+    d.batch = batch;
+    d.wstride = L.enc_size;
+    return d;
 }
 
-// dX = dY W (when dX is wanted); dW += dY^T X; db += the column sums of dY
-static bool gemm_bwd(ndf_hash_model* m, const float* W, const float* X, const float* dY, float* dX,
-                     float* dW, float* db, int c_out, int c_in, int64_t B) {
-    cudaStream_t s = m->ctx->stream;
-    if (dX && gemm_f32_nn(s, dY, W, dX, B, c_in, c_out) != cudaSuccess) return false;
-    if (gemm_f32_tn_acc(s, dY, X, dW, c_out, c_in, B, m->gemm_work) != cudaSuccess) return false;
-    m->ctx->launches += 5;
-    return colsum_f32_acc(s, dY, db, B, c_out, m->gemm_work) == cudaSuccess;
+static DenseLayer dec_layer(const ndf_hash_model* m, int k, int64_t rows) {
+    const HashLayout& L = m->Ly;
+    DenseLayer d;
+    d.W = m->params + L.dw[k];
+    d.b = m->params + L.db[k];
+    d.cin = k == 0 ? L.ddec : L.c;
+    d.cout = L.c;
+    d.rows = rows;
+    return d;
 }
 
-// encoder e over the positions pos[B][3]: fills x0 / pre / post of side s
-static cudaError_t encode_side(ndf_hash_model* m, int e, int s, const float* pos, int64_t B) {
+static const float* post_or_null(const float* pre, const float* post) { return pre == post ? nullptr : post; }
+
+// The encoder chain over rows row0 .. row0 + rows of the workspace: rows [0, B) of them take
+// their positions from pos0, the rest from pos1; `batch` weight sets from encoder e on share the
+// rows evenly.  Leaves x0, pre and post of the rows.
+static cudaError_t encode_rows(ndf_hash_model* m, int e, int batch, const float* pos0, const float* pos1,
+                               int64_t B, int64_t rows, int64_t row0) {
     const HashLayout& L = m->Ly;
     ndf_ctx* ctx = m->ctx;
-    const float* enc = m->params + L.enc_size * e;
-    hash_embed_kernel<<<blocks_for(B, 128), 128, 0, ctx->stream>>>(pos, B, enc, embed_args(L),
-                                                                   m->x0[s]);
+    const float* enc0 = m->params + L.enc_size * e;
+    float* x0 = m->x0 + row0 * L.din;
+    hash_embed_kernel<<<blocks_for(rows, kEmbedRows), 256, sizeof(float) * kEmbedRows * (size_t)(L.din | 1),
+                        ctx->stream>>>(pos0, pos1, B, rows, enc0, enc0 + L.enc_size * (batch - 1), embed_args(L), x0);
     ctx->launches++;
-    const float* in = m->x0[s];
-    for (int k = 0; k < L.le; ++k) {
-        const int cin = k == 0 ? L.din : L.c;
-        if (!gemm_fwd(m, enc + L.ew[k], in, m->pre_e[s][k], L.c, cin, B))
-            return cudaErrorUnknown;
-        bias_act_kernel<<<blocks_for((int64_t)L.c * B), 256, 0, ctx->stream>>>(
-            m->pre_e[s][k], enc + L.eb[k], L.c, B, k < L.le - 1 ? L.act : -1, m->post_e[s][k]);
+    cudaError_t st = cudaGetLastError();
+    const float* in = x0;
+    for (int k = 0; k < L.le && st == cudaSuccess; ++k) {
+        float *pre = m->pre_e[k] + row0 * L.c, *post = m->post_e[k] + row0 * L.c;
+        st = dense_forward(ctx->stream, enc_layer(m, e, k, rows / batch, batch), in, pre,
+                           const_cast<float*>(post_or_null(pre, post)), L.act);
         ctx->launches++;
-        in = m->post_e[s][k];
+        in = post;
     }
-    return cudaGetLastError();
+    return st;
 }
 
-// the latent of side s: the last encoder layer, or the embedding (grid-only)
-static const float* latent(const ndf_hash_model* m, int s) {
-    return m->Ly.le > 0 ? m->post_e[s][m->Ly.le - 1] : m->x0[s];
+// the latents: the last encoder layer, or the embedding (grid-only), from row row0 on
+static const float* latent(const ndf_hash_model* m, int64_t row0) {
+    return (m->Ly.le > 0 ? m->post_e[m->Ly.le - 1] : m->x0) + row0 * m->Ly.dlat;
 }
 
-// decoder over m->z; raw outputs in pre_d[ld-1]
-static cudaError_t decode_z(ndf_hash_model* m, int64_t B) {
+// decoder over m->z: the hidden layers, then the output layer (y; with target the loss and the
+// gradient of the output layer's input in m->ga, its own gradients' partial sums listed)
+static cudaError_t decode_z(ndf_hash_model* m, int64_t B, const float* target, float* y, float* grad) {
     const HashLayout& L = m->Ly;
     ndf_ctx* ctx = m->ctx;
     const float* in = m->z;
-    for (int k = 0; k < L.ld; ++k) {
-        const int cout = k == L.ld - 1 ? 1 : L.c, cin = k == 0 ? L.ddec : L.c;
-        if (!gemm_fwd(m, m->params + L.dw[k], in, m->pre_d[k], cout, cin, B))
-            return cudaErrorUnknown;
-        bias_act_kernel<<<blocks_for((int64_t)cout * B), 256, 0, ctx->stream>>>(
-            m->pre_d[k], m->params + L.db[k], cout, B, k < L.ld - 1 ? L.act : -1, m->post_d[k]);
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < L.ld - 1 && e == cudaSuccess; ++k) {
+        e = dense_forward(ctx->stream, dec_layer(m, k, B), in, m->pre_d[k], m->post_d[k], L.act);
         ctx->launches++;
         in = m->post_d[k];
     }
+    if (e != cudaSuccess) return e;
+    const int k = L.ld - 1, cin = k == 0 ? L.ddec : L.c;
+    const int64_t chunk = target ? out_chunk(B) : kOutRows;
+    const unsigned blocks = (unsigned)((B + chunk - 1) / chunk);
+    float* part = nullptr;
+    if (target) {
+        GradSums& g = m->sums;
+        part = g.take((int64_t)blocks * (cin + 1));
+        if (!part) return cudaErrorInvalidValue;  // the list is empty here and holds one layer
+        // weights and bias are adjacent in the parameters: one segment
+        g.seg[g.count++] = {part, grad + L.dw[k], cin + 1, (int)blocks, 1};
+    }
+    hash_out_kernel<<<blocks, 256, 0, ctx->stream>>>(in, m->params + L.dw[k], m->params + L.db[k], cin, B, chunk,
+                                                     m->measure, target, y, k > 0 ? m->pre_d[k - 1] : nullptr, L.act, m->ga, part,
+                                                     m->loss);
+    ctx->launches++;
     return cudaGetLastError();
 }
 
-// full forward (and, with target, the L1 loss, gradient into m->grad)
+// full forward (and, with target, the L1 loss and the gradient, added to grad[total])
 static cudaError_t hash_forward_backward(ndf_hash_model* m, const float* pr, const float* pq,
-                                         const float* target, int64_t B, float* y) {
+                                         const float* target, int64_t B, float* y, float* grad) {
     const HashLayout& L = m->Ly;
     ndf_ctx* ctx = m->ctx;
-    const int eq = L.n_enc - 1;
-    cudaError_t e = encode_side(m, 0, 0, pr, B);
-    if (e == cudaSuccess) e = encode_side(m, eq, 1, pq, B);
+    cudaStream_t s = ctx->stream;
+    GradSums& g = m->sums;
+    g.count = 0;
+    g.used = 0;
+    const int batch = L.n_enc;  // a shared encoder sees both sides' rows at once
+    cudaError_t e = encode_rows(m, 0, batch, pr, pq, B, 2 * B, 0);
     if (e != cudaSuccess) return e;
-    const float* zr = latent(m, 0);
-    const float* zq = latent(m, 1);
-    merge_kernel<<<blocks_for((int64_t)L.dlat * B), 256, 0, ctx->stream>>>(zr, L.dlat, zq, L.dlat, B,
-                                                                           L.merge, m->z);
+    const float *zr = latent(m, 0), *zq = latent(m, B);
+    merge_kernel<<<blocks_for((int64_t)L.dlat * B), 256, 0, s>>>(zr, L.dlat, zq, L.dlat, B, L.merge, m->z);
     ctx->launches++;
-    if ((e = decode_z(m, B)) != cudaSuccess) return e;
-    out_loss_kernel<<<blocks_for(B), 256, 0, ctx->stream>>>(m->pre_d[L.ld - 1], target, B,
-                                                             m->measure, y, m->graw, m->loss);
-    ctx->launches++;
-    if (!target) return cudaGetLastError();
-    // ---- backward: decoder (ping-pong ga / gb), merge, then each encoder side
-    const float* g = m->graw;  // dL/d(raw output), [1][B]
-    float* pp[2] = {m->ga, m->gb};
-    int cur = 0;
-    for (int k = L.ld - 1; k >= 0; --k) {
-        const int cout = k == L.ld - 1 ? 1 : L.c, cin = k == 0 ? L.ddec : L.c;
-        const float* in = k == 0 ? m->z : m->post_d[k - 1];
-        float* gin = pp[cur];
-        if (!gemm_bwd(m, m->params + L.dw[k], in, g, gin, m->grad + L.dw[k], m->grad + L.db[k],
-                      cout, cin, B))
-            return cudaErrorUnknown;
-        if (k > 0) {
-            dact_mul_kernel<<<blocks_for((int64_t)L.c * B), 256, 0, ctx->stream>>>(
-                gin, m->pre_d[k - 1], (int64_t)L.c * B, L.act);
-            ctx->launches++;
-        }
-        g = gin;
-        cur ^= 1;
+    if ((e = decode_z(m, B, target, y, grad)) != cudaSuccess || !target) return e;
+    // ---- backward: decoder (ping-pong ga / gb), merge, then the encoder chain
+    float *cur = m->ga, *other = m->gb;
+    for (int k = L.ld - 2; k >= 0; --k) {
+        e = dense_backward(s, dec_layer(m, k, B), k == 0 ? m->z : m->post_d[k - 1], cur, other, 0,
+                           k > 0 ? m->pre_d[k - 1] : nullptr, L.act, grad + L.dw[k], grad + L.db[k], g,
+                           &ctx->launches);
+        if (e != cudaSuccess) return e;
+        std::swap(cur, other);
     }
-    merge_backward_kernel<<<blocks_for((int64_t)L.dlat * B), 256, 0, ctx->stream>>>(
-        g, zr, zq, L.dlat, B, L.merge, m->gr, m->gq);
+    merge_backward_kernel<<<blocks_for((int64_t)L.dlat * B), 256, 0, s>>>(cur, zr, zq, L.dlat, B, L.merge, m->gl,
+                                                                          m->gl + B * L.dlat);
     ctx->launches++;
-    for (int s = 0; s < 2; ++s) {
-        const int enc_i = s == 0 ? 0 : eq;  // a shared encoder accumulates both sides
-        const float* enc = m->params + L.enc_size * enc_i;
-        float* genc = m->grad + L.enc_size * enc_i;
-        const float* gs = s == 0 ? m->gr : m->gq;
-        int t = 0;
-        for (int k = L.le - 1; k >= 0; --k) {
-            const int cin = k == 0 ? L.din : L.c;
-            const float* in = k == 0 ? m->x0[s] : m->post_e[s][k - 1];
-            float* gin = pp[t];
-            if (!gemm_bwd(m, enc + L.ew[k], in, gs, gin, genc + L.ew[k], genc + L.eb[k],
-                          L.c, cin, B))
-                return cudaErrorUnknown;
-            if (k > 0) {
-                dact_mul_kernel<<<blocks_for((int64_t)L.c * B), 256, 0, ctx->stream>>>(
-                    gin, m->pre_e[s][k - 1], (int64_t)L.c * B, L.act);
-                ctx->launches++;
-            }
-            gs = gin;
-            t ^= 1;
-        }
-        hash_embed_backward_kernel<<<blocks_for(B, 128), 128, 0, ctx->stream>>>(
-            s == 0 ? pr : pq, B, gs, embed_args(L), genc);
-        ctx->launches++;
+    const float* gs = m->gl;
+    cur = m->ga;
+    other = m->gb;
+    const int col0 = 3 + 6 * L.L;  // positions and Fourier features have no parameters behind them
+    for (int k = L.le - 1; k >= 0; --k) {
+        e = dense_backward(s, enc_layer(m, 0, k, 2 * B / batch, batch), k == 0 ? m->x0 : m->post_e[k - 1], gs, cur,
+                           k == 0 ? col0 : 0, k > 0 ? m->pre_e[k - 1] : nullptr, L.act, grad + L.ew[k],
+                           grad + L.eb[k], g, &ctx->launches);
+        if (e != cudaSuccess) return e;
+        gs = cur;
+        std::swap(cur, other);
     }
-    return cudaGetLastError();
+    const bool grid_only = L.le == 0;
+    hash_embed_backward_kernel<<<dim3(blocks_for(2 * B), (unsigned)L.levels), 256, 0, s>>>(
+        pr, pq, B, 2 * B, grid_only ? gs + col0 : gs, grid_only ? L.din : L.din - col0, embed_args(L), grad,
+        grad + L.enc_size * (L.n_enc - 1));
+    ctx->launches++;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return grad_sums_flush(s, g, &ctx->launches);
 }
 
 
@@ -558,25 +670,22 @@ static cudaError_t hash_fp32_decode(ndf_hash_model* m, int64_t ref_idx, float* d
     const int64_t chunk = std::min<int64_t>(N, 65536);
     cudaError_t e = hash_workspace(m, chunk);
     if (e != cudaSuccess) return e;
+    // rows of the workspace: the reference in row 0, a chunk of queries from row `chunk` on
     vertex_positions_kernel<<<1, 32, 0, ctx->stream>>>(ref_idx, 1, m->X, m->Y, m->Z, m->pos);
     ctx->launches++;
-    e = encode_side(m, 0, 0, m->pos, 1);
+    e = encode_rows(m, 0, 1, m->pos, m->pos, 1, 1, 0);
     const float* zr = latent(m, 0);
+    float* pq = m->pos + 3 * chunk;
     for (int64_t v0 = 0; v0 < N && e == cudaSuccess; v0 += chunk) {
         const int64_t n = std::min(chunk, N - v0);
-        vertex_positions_kernel<<<blocks_for(n), 256, 0, ctx->stream>>>(v0, n, m->X, m->Y, m->Z,
-                                                                         m->pos + 3);
+        vertex_positions_kernel<<<blocks_for(n), 256, 0, ctx->stream>>>(v0, n, m->X, m->Y, m->Z, pq);
         ctx->launches++;
-        e = encode_side(m, L.n_enc - 1, 1, m->pos + 3, n);
+        e = encode_rows(m, L.n_enc - 1, 1, pq, pq, n, n, chunk);
         if (e != cudaSuccess) break;
         merge_kernel<<<blocks_for((int64_t)L.dlat * n), 256, 0, ctx->stream>>>(
-            zr, 0, latent(m, 1), L.dlat, n, L.merge, m->z);
+            zr, 0, latent(m, chunk), L.dlat, n, L.merge, m->z);
         ctx->launches++;
-        if ((e = decode_z(m, n)) != cudaSuccess) break;
-        out_loss_kernel<<<blocks_for(n), 256, 0, ctx->stream>>>(m->pre_d[L.ld - 1], nullptr, n, m->measure,
-                                                                 dev_out + v0, nullptr, nullptr);
-        ctx->launches++;
-        e = cudaGetLastError();
+        e = decode_z(m, n, nullptr, dev_out + v0, nullptr);
     }
     return e;
 }
@@ -682,7 +791,7 @@ ndf_status ndf_hash_model_create(ndf_ctx* ctx, const ndf_hash_arch* arch, int me
 void ndf_hash_model_free(ndf_hash_model* m) {
     if (!m) return;
     if (m->ctx) cudaStreamSynchronize(m->ctx->stream);
-    void* ps[] = {m->params, m->grad, m->m, m->v, m->ws, m->gemm_work, m->tc_w, m->tc_bias,
+    void* ps[] = {m->params, m->grad, m->m, m->v, m->ws, m->sums.work, m->tc_w, m->tc_bias,
                   m->tc_zr, m->tc_lat, m->tc_ftab};
     for (void* q : ps)
         if (q) cudaFree(q);
@@ -708,23 +817,25 @@ ndf_status ndf_hash_model_set_params(ndf_hash_model* m, const float* in) {
     return e == cudaSuccess ? NDF_OK : cuda_fail(m->ctx, e, "hash params upload");
 }
 
-// positions / targets / outputs may be host or device; staged through the workspace
+static cudaError_t hash_adam(ndf_hash_model* m, const float* grad, float lr) {
+    ++m->t;
+    ++m->ver;
+    const float c1 = 1.0f - powf(0.9f, (float)m->t), c2 = 1.0f - powf(0.999f, (float)m->t);
+    hash_adam_kernel<<<blocks_for((m->Ly.total + 3) / 4), 256, 0, m->ctx->stream>>>(
+        m->params, grad, m->m, m->v, m->Ly.total, ((uintptr_t)grad & 15) == 0, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
+    m->ctx->launches++;
+    return cudaGetLastError();
+}
+
 // one training step on device batches (no copies, no host synchronisation): the
 // summed |error| of the batch accumulates in m->loss
 static cudaError_t hash_train_step(ndf_hash_model* m, const float* pr, const float* pq,
                                    const float* target, int64_t B, float lr) {
     ndf_ctx* ctx = m->ctx;
     cudaError_t e = cudaMemsetAsync(m->grad, 0, sizeof(float) * (size_t)m->Ly.total, ctx->stream);
-    if (e == cudaSuccess) e = hash_forward_backward(m, pr, pq, target, B, nullptr);
+    if (e == cudaSuccess) e = hash_forward_backward(m, pr, pq, target, B, nullptr, m->grad);
     if (e != cudaSuccess) return e;
-    ++m->t;
-    ++m->ver;
-    const float c1 = 1.0f - powf(0.9f, (float)m->t), c2 = 1.0f - powf(0.999f, (float)m->t);
-    hash_adam_kernel<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(m->params, m->grad, m->m, m->v,
-                                                                m->Ly.total, lr, 0.9f, 0.999f, 1e-8f,
-                                                                c1, c2);
-    ctx->launches++;
-    return cudaGetLastError();
+    return hash_adam(m, m->grad, lr);
 }
 
 ndf_status ndf_hash_model_step(ndf_hash_model* m, const float* pr, const float* pq,
@@ -740,22 +851,16 @@ ndf_status ndf_hash_model_step(ndf_hash_model* m, const float* pr, const float* 
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->pos + 3 * B, pq, pb, cudaMemcpyDefault, ctx->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m->tgt, target, sizeof(float) * B, cudaMemcpyDefault, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->grad, 0, sizeof(float) * (size_t)m->Ly.total, ctx->stream);
+    // a gradient buffer of the caller on this device serves as the step's own (no copy of it)
+    const size_t gb = sizeof(float) * (size_t)m->Ly.total;
+    float* grad = grad_out && device_writable(ctx, grad_out) ? grad_out : m->grad;
+    if (e == cudaSuccess) e = cudaMemsetAsync(grad, 0, gb, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->loss, 0, sizeof(double), ctx->stream);
-    if (e == cudaSuccess) e = hash_forward_backward(m, m->pos, m->pos + 3 * B, m->tgt, B, nullptr);
-    if (e == cudaSuccess && apply) {
-        ++m->t;
-        ++m->ver;
-        const float c1 = 1.0f - powf(0.9f, (float)m->t), c2 = 1.0f - powf(0.999f, (float)m->t);
-        hash_adam_kernel<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(
-            m->params, m->grad, m->m, m->v, m->Ly.total, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
-        ctx->launches++;
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = hash_forward_backward(m, m->pos, m->pos + 3 * B, m->tgt, B, nullptr, grad);
+    if (e == cudaSuccess && apply) e = hash_adam(m, grad, lr);
     double l = 0.0;
-    if (e == cudaSuccess && grad_out)
-        e = cudaMemcpyAsync(grad_out, m->grad, sizeof(float) * (size_t)m->Ly.total, cudaMemcpyDefault,
-                            ctx->stream);
+    if (e == cudaSuccess && grad_out && grad != grad_out)
+        e = cudaMemcpyAsync(grad_out, grad, gb, cudaMemcpyDefault, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&l, m->loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "hash step");
@@ -773,8 +878,8 @@ ndf_status ndf_hash_model_forward(ndf_hash_model* m, const float* pr, const floa
     const size_t pb = sizeof(float) * 3 * (size_t)B;
     e = cudaMemcpyAsync(m->pos, pr, pb, cudaMemcpyDefault, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->pos + 3 * B, pq, pb, cudaMemcpyDefault, ctx->stream);
-    if (e == cudaSuccess) e = hash_forward_backward(m, m->pos, m->pos + 3 * B, nullptr, B, m->graw);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, m->graw, sizeof(float) * B, cudaMemcpyDefault, ctx->stream);
+    if (e == cudaSuccess) e = hash_forward_backward(m, m->pos, m->pos + 3 * B, nullptr, B, m->y, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out, m->y, sizeof(float) * B, cudaMemcpyDefault, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     return e == cudaSuccess ? NDF_OK : cuda_fail(ctx, e, "hash forward");
 }

@@ -95,6 +95,8 @@ void ctx_trim(ndf_ctx* ctx);
 // Returns a field's buffers to the cache (standardised copies are freed) and marks it dead.
 void release_field(ndf_ctx* ctx, Field& f);
 PtrKind pointer_kind(const void* p);
+// a 4-byte-aligned pointer into device memory of the context's own GPU
+bool device_writable(const ndf_ctx* ctx, const void* p);
 
 ndf_status fail(ndf_ctx* ctx, ndf_status st, const char* fmt, ...);
 ndf_status cuda_fail(ndf_ctx* ctx, cudaError_t e, const char* what);
