@@ -696,7 +696,7 @@ cudaError_t mlp_tc_forward(ndf_model* m, int64_t B, float* y) {
     return cudaGetLastError();
 }
 
-cudaError_t mlp_tc_train(ndf_model* m, int64_t B, const float* target) {
+cudaError_t mlp_tc_train(ndf_model* m, int64_t B, const float* target, float* grad) {
     cudaError_t e = set_attrs();
     if (e != cudaSuccess) return e;
     ndf_ctx* ctx = m->ctx;
@@ -723,9 +723,9 @@ cudaError_t mlp_tc_train(ndf_model* m, int64_t B, const float* target) {
     if (grid > tiles) grid = tiles;
     if (grid < 1) grid = 1;
     mlp_train_tc_kernel<<<(unsigned)grid, kTrainThreads, kTrainSmem, s>>>(a);
-    wgrad_reduce_kernel<<<dim3(kHid * kHid / 256, 3), 256, 0, s>>>(m->work.wpart, (int)grid, m->grad,
+    wgrad_reduce_kernel<<<dim3(kHid * kHid / 256, 3), 256, 0, s>>>(m->work.wpart, (int)grid, grad,
                                                                   m->L.W1, m->L.W2, m->L.W3);
-    colsum_reduce_kernel<<<dim3(kHid, kColSums), 128, 0, s>>>(m->work.cpart, (int)grid * 4, m->grad, m->L.b1,
+    colsum_reduce_kernel<<<dim3(kHid, kColSums), 128, 0, s>>>(m->work.cpart, (int)grid * 4, grad, m->L.b1,
                                                               m->L.b2, m->L.b3, m->L.w4, m->L.b4);
     ctx->launches += 3;
     return cudaGetLastError();

@@ -220,7 +220,14 @@ __global__ void __launch_bounds__(256)
     float4* g4 = reinterpret_cast<float4*>(gr);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
         float4 P = __ldcs(p4 + i), M = __ldcs(m4 + i), V = __ldcs(v4 + i);
-        const float4 G = __ldcs(g4 + i);
+        float4 G;
+        if (CLEAR || (i << 2) + 3 < n) {
+            G = __ldcs(g4 + i);
+        } else {  // a caller's buffer ends at n; the padding's gradient is zero
+            const float* g = gr + (i << 2);
+            const int64_t left = n - (i << 2);
+            G = make_float4(g[0], left > 1 ? g[1] : 0.f, left > 2 ? g[2] : 0.f, 0.f);
+        }
         adam4(P, G, M, V, lr, beta1, beta2, eps, c1, c2);
         __stcs(p4 + i, P);
         __stcs(m4 + i, M);
@@ -370,51 +377,60 @@ ndf_status ensure_work(ndf_model* m, int64_t B) {
     return NDF_OK;
 }
 
+cudaError_t model_adam(ndf_model* m, float* grad, bool clear, float lr, float beta1, float beta2, float eps) {
+    ndf_ctx* ctx = m->ctx;
+    cudaStream_t s = ctx->stream;
+    m->t += 1;
+    const float c1 = (float)(1.0 - pow((double)beta1, (double)m->t));
+    const float c2 = (float)(1.0 - pow((double)beta2, (double)m->t));
+    // 64 CTAs per SM, or one thread per group of four parameters if that is fewer
+    const int64_t groups_ctas = ((m->L.total + 3) / 4 + 255) / 256;
+    const unsigned ctas = (unsigned)(groups_ctas < (int64_t)ctx->sm_count * 64 ? groups_ctas
+                                                                               : (int64_t)ctx->sm_count * 64);
+    if (clear)
+        adam_kernel<true><<<ctas, 256, 0, s>>>(m->params, grad, m->m, m->v, m->L.total, m->L.n_grid,
+                                               m->grid_bf, lr, beta1, beta2, eps, c1, c2);
+    else
+        adam_kernel<false><<<ctas, 256, 0, s>>>(m->params, grad, m->m, m->v, m->L.total, m->L.n_grid,
+                                                m->grid_bf, lr, beta1, beta2, eps, c1, c2);
+    refresh_mlp_kernel<<<(3 * kHid * kHid + 255) / 256, 256, 0, s>>>(
+        m->params, m->L.W1, m->L.W2, m->L.W3, m->wbf);
+    ctx->launches += 2;
+    return cudaGetLastError();
+}
+
 cudaError_t model_step(ndf_model* m, const float* pr, const float* pq, const float* target,
                        int64_t B, float lr, float beta1, float beta2, float eps, bool update,
-                       bool keep_grad) {
+                       float* grad_out) {
     ndf_ctx* ctx = m->ctx;
     cudaStream_t s = ctx->stream;
     NetWork& w = m->work;
-    // gradients start from zero every step: Adam clears them as it reads them, so only
-    // after a step that kept its gradient is the buffer cleared here.  The loss sum in
-    // w.loss accumulates across steps (callers zero it).
+    // gradients start from zero every step: Adam clears the model's own buffer as it reads it, so
+    // that one is cleared here only after a step without an update; a buffer of the caller
+    // (grad_out) takes its place in a step that returns the gradient, which then needs no copy
+    // (2.46 GB for the default grid: 0.37 ms of a 3.12 ms step).  The loss sum in w.loss
+    // accumulates across steps (callers zero it).
     cudaError_t e = cudaSuccess;
-    if (!m->grad_zero) {
+    float* grad = grad_out ? grad_out : m->grad;
+    if (grad_out) {
+        e = cudaMemsetAsync(grad_out, 0, (size_t)m->L.total * 4, s);
+    } else if (!m->grad_zero) {
         e = cudaMemsetAsync(m->grad, 0, (((size_t)m->L.total + 3) & ~size_t(3)) * 4, s);
-        if (e != cudaSuccess) return e;
-        m->grad_zero = true;
     }
+    if (e != cudaSuccess) return e;
+    if (!grad_out) m->grad_zero = false;
     const GridDev G = grid_dev(m);
     encode_merge_fwd_kernel<<<(unsigned)((B * kLevels + 255) / 256), 256, 0, s>>>(G, pr, pq, B, w.fr,
                                                                                  w.fq, w.x);
     ctx->launches++;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = mlp_tc_train(m, B, target)) != cudaSuccess) return e;
+    if ((e = mlp_tc_train(m, B, target, grad)) != cudaSuccess) return e;
     encode_bwd_kernel<<<(unsigned)((B * kLevels * 2 * 4 + 255) / 256), 256, 0, s>>>(
-        G, pr, pq, B, w.fr, w.fq, w.dx, m->grad);
+        G, pr, pq, B, w.fr, w.fq, w.dx, grad);
     ctx->launches++;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (update) {
-        m->t += 1;
-        const float c1 = (float)(1.0 - pow((double)beta1, (double)m->t));
-        const float c2 = (float)(1.0 - pow((double)beta2, (double)m->t));
-        // 64 CTAs per SM, or one thread per group of four parameters if that is fewer
-        const int64_t groups_ctas = ((m->L.total + 3) / 4 + 255) / 256;
-        const unsigned ctas = (unsigned)(groups_ctas < (int64_t)ctx->sm_count * 64 ? groups_ctas
-                                                                                   : (int64_t)ctx->sm_count * 64);
-        if (keep_grad)
-            adam_kernel<false><<<ctas, 256, 0, s>>>(m->params, m->grad, m->m, m->v, m->L.total, m->L.n_grid,
-                                                    m->grid_bf, lr, beta1, beta2, eps, c1, c2);
-        else
-            adam_kernel<true><<<ctas, 256, 0, s>>>(m->params, m->grad, m->m, m->v, m->L.total, m->L.n_grid,
-                                                   m->grid_bf, lr, beta1, beta2, eps, c1, c2);
-        refresh_mlp_kernel<<<(3 * kHid * kHid + 255) / 256, 256, 0, s>>>(
-            m->params, m->L.W1, m->L.W2, m->L.W3, m->wbf);
-        ctx->launches += 2;
-        e = cudaGetLastError();
-    }
-    m->grad_zero = update && !keep_grad;
+    if (update) e = model_adam(m, grad, !grad_out, lr, beta1, beta2, eps);
+    if (!grad_out) m->grad_zero = update && e == cudaSuccess;
     return e;
 }
 

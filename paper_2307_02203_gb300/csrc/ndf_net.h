@@ -83,19 +83,22 @@ ndf_status ensure_work(ndf_model* m, int64_t B);
 
 // One step on a batch of device positions (pr, pq: [B][3]) and targets: loss
 // (accumulated in work.loss) and gradients; with update, one Adam step.
-// keep_grad: leave this step's gradient in m->grad after the update (a caller reads it)
+// grad_out (on the model's GPU, 16-byte aligned, L.total floats, apart from the inputs): the
+// step's gradient is built there instead of in m->grad and stays after the update
 cudaError_t model_step(ndf_model* m, const float* pr, const float* pq, const float* target,
                        int64_t B, float lr, float beta1, float beta2, float eps, bool update,
-                       bool keep_grad = false);
+                       float* grad_out = nullptr);
+// the update alone, from grad (cleared as it is read if clear)
+cudaError_t model_adam(ndf_model* m, float* grad, bool clear, float lr, float beta1, float beta2, float eps);
 cudaError_t net_set_attributes();
 cudaError_t model_forward(ndf_model* m, const float* pr, const float* pq, int64_t B, float* out);
 
 // The MLP on tcgen05 (ndf_mlp_tc.cu), over the merged input in m->work.x: the
 // forward alone (y = the network output), and the training pass (the L1 loss sum
 // into m->work.loss, the gradients of the three layers and of the output layer
-// added into m->grad, the input gradient in m->work.dx).
+// added into grad, the input gradient in m->work.dx).
 cudaError_t mlp_tc_forward(ndf_model* m, int64_t B, float* y);
-cudaError_t mlp_tc_train(ndf_model* m, int64_t B, const float* target);
+cudaError_t mlp_tc_train(ndf_model* m, int64_t B, const float* target, float* grad);
 
 // Volume decoding for R references (vertex ids on the device): out[R][N].
 cudaError_t model_infer(ndf_model* m, const int64_t* d_refs, int R, float* out);

@@ -403,11 +403,25 @@ ndf_status ndf_model_step(ndf_model* m, const float* p_ref, const float* p_query
     ndf_status st = stage_batch(m, p_ref, p_query, target, B, &dpr, &dpq, &dt);
     if (st != NDF_OK) return st;
     cudaError_t e = cudaMemsetAsync(m->work.loss, 0, 8, ctx->stream);
-    if (e == cudaSuccess)
-        e = model_step(m, dpr, dpq, dt, B, lr, 0.9f, 0.999f, 1e-8f, update != 0, grad_out != nullptr);
-    if (e == cudaSuccess && grad_out)
-        e = cudaMemcpyAsync(grad_out, m->grad, (size_t)m->L.total * 4, cudaMemcpyDefault,
-                            ctx->stream);
+    // a 16-byte-aligned gradient buffer of the caller on this device, apart from the batch that
+    // the step reads, is used as the step's gradient; any other gets a copy of the model's own
+    const size_t gb = (size_t)m->L.total * 4;
+    auto apart = [&](const void* p, size_t n) {
+        return (uintptr_t)p + n <= (uintptr_t)grad_out || (uintptr_t)grad_out + gb <= (uintptr_t)p;
+    };
+    const bool direct = grad_out && ((uintptr_t)grad_out & 15) == 0 && device_writable(ctx, grad_out) &&
+                        apart(dpr, (size_t)B * 12) && apart(dpq, (size_t)B * 12) && apart(dt, (size_t)B * 4);
+    if (e == cudaSuccess && grad_out && !direct && update) {
+        // the gradient first, copied before the update clears it
+        e = model_step(m, dpr, dpq, dt, B, lr, 0.9f, 0.999f, 1e-8f, false, nullptr);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(grad_out, m->grad, gb, cudaMemcpyDefault, ctx->stream);
+        if (e == cudaSuccess) e = model_adam(m, m->grad, true, lr, 0.9f, 0.999f, 1e-8f);
+        m->grad_zero = e == cudaSuccess;
+    } else if (e == cudaSuccess) {
+        e = model_step(m, dpr, dpq, dt, B, lr, 0.9f, 0.999f, 1e-8f, update != 0, direct ? grad_out : nullptr);
+        if (e == cudaSuccess && grad_out && !direct)
+            e = cudaMemcpyAsync(grad_out, m->grad, gb, cudaMemcpyDefault, ctx->stream);
+    }
     double loss = 0.0;
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(&loss, m->work.loss, 8, cudaMemcpyDeviceToHost, ctx->stream);
