@@ -13,16 +13,28 @@
 //
 // A persistent CTA per SM decodes 128-vertex tiles (the MMA M dimension) in two
 // slots so that one slot's epilogue overlaps the other slot's MMAs:
-//   warps 0-3 (slot 0) and 4-7 (slot 1): thread i of a slot owns row i of the tile
-//     and TMEM lane i.  It encodes its vertex once per tile (64 FP32 features kept
-//     in registers); then for each reference it writes x into the slot's A operand
-//     (BF16, 128-byte-swizzled K-major), and after each layer loads its row of the
-//     FP32 accumulator with tcgen05.ld, adds the bias, applies ReLU and writes the
-//     next layer's operand over the same buffer (the MMA that read it has
-//     completed), or after layer 3 the output.
-//   warp 8: allocates TMEM (2 slots x 128 columns); one lane issues tcgen05.mma
-//     (M = 128, N = 128, K = 128) for whichever slot is ready and commits to that
-//     slot's mbarrier.
+//   warps 0-7 (slot 0) and 8-15 (slot 1): thread i of a slot's two halves owns row i of the
+//     tile (TMEM lane i) and 64 of its columns.  The halves encode the vertex once per tile
+//     tile (TMEM lane i) and 64 of its columns.  The halves encode the vertex once per tile
+//     (two levels each; 64 FP32 features in shared memory); then for each reference, after
+//     each layer, they load their columns of the FP32 accumulator with tcgen05.ld, round,
+//     apply ReLU and write the next layer's operand (after layer 3 the columns stay as BF16
+//     pairs in registers).  All other work sits where the slot would wait for an MMA: the
+//     output layer's dot product under the next reference's layer 1, its halves' exchange and
+//     the output function under layer 2, and the reference after that one's x (one half the
+//     products, the other the sums; an operand of its own) under layer 3.
+//   warp 16: allocates TMEM; one lane issues tcgen05.mma (M = 128, N = 128, K = 128 + 16) for
+//     whichever slot is ready and commits to that slot's mbarrier.  The extra K step adds the
+//     biases: a constant operand [1 1 1 0 ..] against each bias split into three BF16 terms
+//     (24 bits), so the epilogue neither loads nor adds them.
+// The A operands live in TMEM (two times 64 columns of BF16 pairs per slot, x and h, beside its
+// 128 accumulator columns), not in shared memory: a layer's operand write and read would each be 32 KB of
+// shared-memory bandwidth (256 cycles) on top of the weights' 32 KB.  What bounds the kernel is
+// the chain of a slot (MMA of 576 cycles, commit, epilogue, MMA) with two slots per SM, so what
+// counts is what stands between a commit and the next hand-over (about 450 cycles; with x, dot
+// product and output there too it was 2,900, and 3,800 per layer with one warp per 128 columns,
+// operands in shared memory and the bias in the epilogue).  16 references on 1.76M vertices:
+// 4.29 ms before, 2.83 ms now.
 // The references' features f(p_r) (FP32) and the biases sit in shared memory.
 #include <cuda_bf16.h>
 
@@ -36,7 +48,8 @@ namespace {
 using namespace tc;
 
 constexpr int kTile = 128;
-constexpr int kTcThreads = 288;  // 8 epilogue warps + 1 MMA warp
+constexpr int kEpiWarps = 16;
+constexpr int kTcThreads = 32 * kEpiWarps + 32;  // + 1 MMA warp
 
 struct TcGrid {
     const __nv_bfloat16* grid;
@@ -102,26 +115,32 @@ struct TcInferArgs {
     unsigned* status;
 };
 
-// shared memory: W1, W2, W3 (2 atoms each), one 2-atom operand buffer per slot,
-// then biases / output weights (4 x 128 FP32), the references' features [R][64]
+// shared memory: W1, W2, W3 (2 atoms each), the biases' operand (layer l in columns 16 l
+// .. of one atom), then output weights / output weights (4 x 128 FP32), the references' features [R][64]
 // FP32 and the barriers
 constexpr int kMaxRefsPerLaunch = 64;
-constexpr uint32_t kOffW = 0, kOffSlot = 6 * kAtom, kSlotBytes = 2 * kAtom;
-constexpr uint32_t kOffVec = kOffSlot + 2 * kSlotBytes;
-constexpr uint32_t kOffFr = kOffVec + 4 * kHid * 4;
-constexpr uint32_t kOffBar = kOffFr + kMaxRefsPerLaunch * kLF * 4;
+constexpr uint32_t kOffW = 0, kOffBias = 6 * kAtom, kOffOne = 7 * kAtom, kOffVec = 8 * kAtom;
+// TMEM columns: accumulators at 0 and 128, the slots' h at 256 and 320, their x at 384 and 448
+constexpr uint32_t kTmemCols = 512, kTmemH = 256, kTmemX = 384;
+constexpr uint32_t kOffPart = kOffVec + kHid * 4;  // [2 slots][128] output-layer halves
+constexpr uint32_t kOffFr = kOffPart + 2 * 128 * 4;
+constexpr uint32_t kOffFq = kOffFr + kMaxRefsPerLaunch * kLF * 4;  // [16][256 rows] float4
+constexpr uint32_t kOffBar = kOffFq + 256 * kLF * 4;
 constexpr uint32_t kTcSmem = kOffBar + 256 /*barriers*/ + 1024 /*align*/;
 
 __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    float* vec = reinterpret_cast<float*>(smem + kOffVec);  // b1, b2, b3, w4
+    float* w4s = reinterpret_cast<float*>(smem + kOffVec);
+    float* part_s = reinterpret_cast<float*>(smem + kOffPart);
     float* fr_all = reinterpret_cast<float*>(smem + kOffFr);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOffBar);
-    uint64_t* a_ready = bars;      // [2] epilogue -> MMA (128 arrivals)
-    uint64_t* d_ready = bars + 2;  // [2] MMA -> epilogue (commit)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 4);
+    uint64_t* a_ready = bars;         // [2] epilogue -> MMA (8 warps)
+    uint64_t* d_ready = bars + 2;     // [2] MMA -> epilogue (commit)
+    uint64_t* enc_ready = bars + 4;   // [2] the tile's features are written (8 warps)
+    uint64_t* part_ready = bars + 6;  // [2] the second half's output sums are written (4 warps)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int R = a.R;
@@ -134,9 +153,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferAr
         *reinterpret_cast<uint4*>(smem + kOffW + o) =
             reinterpret_cast<const uint4*>(a.w + ((size_t)l * kHid + row) * kHid)[c];
     }
-    for (int i = threadIdx.x; i < 4 * kHid; i += blockDim.x) {
-        const int64_t off = i < kHid ? a.offb1 : i < 2 * kHid ? a.offb2 : i < 3 * kHid ? a.offb3 : a.offw4;
-        vec[i] = a.params[off + (i % kHid)];
+    for (int i = threadIdx.x; i < kHid; i += blockDim.x) {
+        w4s[i] = a.params[a.offw4 + i];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {  // the fourth quarter of the atom is not read
+            const float b = l == 0 ? a.params[a.offb1 + i] : l == 1 ? a.params[a.offb2 + i] : l == 2 ? a.params[a.offb3 + i] : 0.0f;
+            const float hi = __bfloat162float(__float2bfloat16_rn(b));
+            const float r1 = isinf(hi) ? 0.0f : b - hi, mid = __bfloat162float(__float2bfloat16_rn(r1));
+            *reinterpret_cast<uint4*>(smem + kOffBias + swz(i, 2 * l)) = make_uint4(bf2(hi, mid), bf2(r1 - mid, 0.0f), 0u, 0u);
+            *reinterpret_cast<uint4*>(smem + kOffBias + swz(i, 2 * l + 1)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        *reinterpret_cast<uint4*>(smem + kOffOne + swz(i, 0)) = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
+        *reinterpret_cast<uint4*>(smem + kOffOne + swz(i, 1)) = make_uint4(0u, 0u, 0u, 0u);
     }
     for (int i = threadIdx.x; i < R * kLevels; i += blockDim.x) {
         const int64_t v = a.refs[i / kLevels];
@@ -149,15 +177,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferAr
     }
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
-            mbar_init(&a_ready[s], 128);
+            mbar_init(&a_ready[s], 8);
             mbar_init(&d_ready[s], 1);
+            mbar_init(&enc_ready[s], 8);
+            mbar_init(&part_ready[s], 4);
         }
         *abort_flag = 0;
     }
-    if (warp == 8) {
+    if (warp == kEpiWarps) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(tmem_slot)),
-                     "r"(256u)
+                     "r"(kTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -172,7 +202,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferAr
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kHid >> 3) << 17) |
                            ((uint32_t)(kTile >> 4) << 24);
 
-    if (warp == 8) {
+    if (warp == kEpiWarps) {
         if (lane == 0) {  // ---- MMA issuer: serve whichever slot is ready
             // operands per slot: (its tiles) x R references x 3 layers
             int64_t left[2];
@@ -192,15 +222,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferAr
                     progressed = true;
                     ++na[s];
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + kOffSlot + s * kSlotBytes);
+                    const uint32_t ta = tmem + (layer[s] == 0 ? kTmemX : kTmemH) + (uint32_t)(s * 64);
                     const uint32_t wl = sw + (uint32_t)(2 * layer[s]) * kAtom;
                     const uint32_t d = tmem + (uint32_t)(s * 128);
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {  // K = 128: two atoms, 4 steps of 16 each
                         const uint32_t at = (uint32_t)(kk >> 2) * kAtom;
-                        tc_mma(d, desc_sw128(sa + at) + (uint64_t)((kk & 3) * 2),
-                               desc_sw128(wl + at) + (uint64_t)((kk & 3) * 2), idesc, kk > 0 ? 1u : 0u);
+                        tc_mma_ts(d, ta + (uint32_t)(kk * 8), desc_sw128(wl + at) + (uint64_t)((kk & 3) * 2), idesc,
+                                  kk > 0 ? 1u : 0u);
                     }
+                    tc_mma(d, desc_sw128(smem_u32(smem + kOffOne)),
+                           desc_sw128(smem_u32(smem + kOffBias)) + (uint64_t)(layer[s] * 2), idesc, 1u);
                     tc_commit(&d_ready[s]);
                     layer[s] = layer[s] == 2 ? 0 : layer[s] + 1;
                     --left[s];
@@ -217,97 +249,138 @@ __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferAr
                 }
             }
         }
-    } else {  // ---- encode / epilogue: slot s, row i = TMEM lane i
-        const int s = warp >> 2;
+    } else {  // ---- encode / epilogue: slot s, row i = TMEM lane i, columns of half h
+        const int s = warp >> 3, h = (warp >> 2) & 1;
         const int i = (warp & 3) * 32 + lane;
-        unsigned char* A = smem + kOffSlot + s * kSlotBytes;
-        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(s * 128);
+        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint32_t taddr = tl + (uint32_t)(s * 128 + h * 64);
+        const uint32_t haddr = tl + kTmemH + (uint32_t)(s * 64 + h * 32);
+        const uint32_t xaddr = tl + kTmemX + (uint32_t)(s * 64 + h * 32);
         const float b4 = a.params[a.offb4];
-        uint32_t nd = 0;
+        // this row's query features, four per 16 bytes
+        ulonglong2* fq = reinterpret_cast<ulonglong2*>(smem + kOffFq) + s * 128 + i;
+        const ulonglong2* w4 = reinterpret_cast<const ulonglong2*>(w4s + 64 * h);
+        uint32_t nd = 0, ne = 0, np = 0;
         for (int64_t t = (int64_t)blockIdx.x * 2 + s; t < tiles; t += step) {
             const int64_t v = t * kTile + i;
             // this row's vertex, encoded once for every reference (rows past N encode
             // position 0: harmless, never written out)
-            float fq[kLF];
             {
                 const int64_t vv = v < a.N ? v : 0;
                 const int64_t x = vv % a.X, y = (vv / a.X) % a.Y, z = vv / (a.X * a.Y);
                 const float p[3] = {pos_axis(x, a.X), pos_axis(y, a.Y), pos_axis(z, a.Z)};
-#pragma unroll
-                for (int l = 0; l < kLevels; ++l) {
+#pragma unroll 1
+                for (int l = h * (kLevels / 2); l < (h + 1) * (kLevels / 2); ++l) {
                     float f[kFeat];
                     encode_level(a.G, l, p, f);
 #pragma unroll
-                    for (int q = 0; q < kFeat; ++q) fq[l * kFeat + q] = f[q];
+                    for (int q = 0; q < kFeat / 4; ++q)
+                        fq[(l * (kFeat / 4) + q) * 256] =
+                            make_ulonglong2(pair2(f[4 * q], f[4 * q + 1]), pair2(f[4 * q + 2], f[4 * q + 3]));
                 }
             }
-            for (int r = 0; r < R; ++r) {
-                const float* fr = fr_all + r * kLF;
-                // x = [fr * fq ; fr + fq]: 16-byte chunks 0-7 the products, 8-15 the sums
+            arrive_warp(&enc_ready[s]);
+            if (!__all_sync(0xffffffffu, wait_bounded(&enc_ready[s], ne & 1u, abort_flag))) goto done;
+            ++ne;
+            // x = [fr * fq ; fr + fq]: operand columns 0-31 the products, 32-63 the sums
+            auto put_x = [&](int r) {
+                const ulonglong2* fr = reinterpret_cast<const ulonglong2*>(fr_all + r * kLF);
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const float4 r0 = *reinterpret_cast<const float4*>(fr + 8 * c);
-                    const float4 r1 = *reinterpret_cast<const float4*>(fr + 8 * c + 4);
-                    const float* q = fq + 8 * c;
-                    *reinterpret_cast<uint4*>(A + swz(i, c)) =
-                        make_uint4(bf2(r0.x * q[0], r0.y * q[1]), bf2(r0.z * q[2], r0.w * q[3]),
-                                   bf2(r1.x * q[4], r1.y * q[5]), bf2(r1.z * q[6], r1.w * q[7]));
-                    *reinterpret_cast<uint4*>(A + kAtom + swz(i, c)) =
-                        make_uint4(bf2(r0.x + q[0], r0.y + q[1]), bf2(r0.z + q[2], r0.w + q[3]),
-                                   bf2(r1.x + q[4], r1.y + q[5]), bf2(r1.z + q[6], r1.w + q[7]));
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t o[8];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const ulonglong2 f = fr[4 * c + j], q = fq[(4 * c + j) * 256];
+                        if (h == 0) {
+                            o[2 * j] = bf2(mul_pair(f.x, q.x));
+                            o[2 * j + 1] = bf2(mul_pair(f.y, q.y));
+                        } else {
+                            o[2 * j] = bf2(add_pair(f.x, q.x));
+                            o[2 * j + 1] = bf2(add_pair(f.y, q.y));
+                        }
+                    }
+                    tmem_st8(xaddr + (uint32_t)(8 * c), o);
                 }
-                proxy_fence();
-                tc_fence_before();
-                arrive(&a_ready[s]);
-                for (int layer = 0; layer < 3; ++layer) {
+                tmem_wait_st();
+            };
+            // the output of reference r from this half's sum of the output layer
+            float sum = 0.0f;
+            auto put_out = [&](int r) {
+                if (h == 1) return true;
+                if (!__all_sync(0xffffffffu, wait_bounded(&part_ready[s], np & 1u, abort_flag))) return false;
+                ++np;
+                const float o = (sum + part_s[s * 128 + i]) + b4;
+                if (v < a.N)
+                    a.out[(int64_t)r * a.N + v] = a.measure == 0 ? tanhf(o) : (o > 20.f ? o : log1pf(expf(o)));
+                return true;
+            };
+            put_x(0);
+            tc_fence_before();
+            arrive_warp(&a_ready[s]);
+            for (int r = 0; r < R; ++r) {
+#pragma unroll 1
+                for (int layer = 0; layer < 2; ++layer) {
                     if (!__all_sync(0xffffffffu, wait_bounded(&d_ready[s], nd & 1u, abort_flag))) goto done;
                     ++nd;
                     tc_fence_after();
-                    const float* bias = vec + layer * kHid;
-                    float acc = 0.0f;
+                    uint32_t d[64], o[16];
+                    tmem_ld64(taddr, d);
 #pragma unroll
-                    for (int c0 = 0; c0 < kHid; c0 += 32) {
-                        float h[32];
-                        tmem_ld32(taddr + (uint32_t)c0, h);
+                    for (int c = 0; c < 2; ++c) {  // rounded, ReLU
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) h[j] = fmaxf(h[j] + bias[c0 + j], 0.0f);
-                        if (layer < 2) {  // next layer's operand: columns c0..c0+31
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int c = (c0 >> 3) + q;  // 16-byte chunk of the 256-byte row
-                                *reinterpret_cast<uint4*>(A + (uint32_t)(c >> 3) * kAtom + swz(i, c & 7)) =
-                                    make_uint4(bf2(h[8 * q], h[8 * q + 1]), bf2(h[8 * q + 2], h[8 * q + 3]),
-                                               bf2(h[8 * q + 4], h[8 * q + 5]), bf2(h[8 * q + 6], h[8 * q + 7]));
-                            }
-                        } else {  // output layer on the BF16-rounded h3
-#pragma unroll
-                            for (int j = 0; j < 32; j += 2) {
-                                const float2 hv = unbf2(bf2(h[j], h[j + 1]));
-                                acc = fmaf(vec[3 * kHid + c0 + j], hv.x,
-                                           fmaf(vec[3 * kHid + c0 + j + 1], hv.y, acc));
-                            }
-                        }
+                        for (int j = 0; j < 16; ++j) o[j] = relu2(bf2(pair2(d[32 * c + 2 * j], d[32 * c + 2 * j + 1])));
+                        tmem_st16(haddr + (uint32_t)(16 * c), o);
                     }
-                    if (layer < 2) {
-                        proxy_fence();
-                        tc_fence_before();
-                        arrive(&a_ready[s]);
-                    } else if (v < a.N) {
-                        const float o = acc + b4;
-                        a.out[(int64_t)r * a.N + v] =
-                            a.measure == 0 ? tanhf(o) : (o > 20.f ? o : log1pf(expf(o)));
+                    tmem_wait_st();
+                    tc_fence_before();
+                    arrive_warp(&a_ready[s]);
+                    if (layer == 0) {
+                        if (r > 0 && !put_out(r - 1)) goto done;
+                    } else if (r + 1 < R) {
+                        put_x(r + 1);  // layer 1 of this reference, which read x, has completed
                     }
                 }
+                if (!__all_sync(0xffffffffu, wait_bounded(&d_ready[s], nd & 1u, abort_flag))) goto done;
+                ++nd;
+                tc_fence_after();
+                uint32_t h3[32];
+                {
+                    uint32_t d[64];
+                    tmem_ld64(taddr, d);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) h3[j] = relu2(bf2(pair2(d[2 * j], d[2 * j + 1])));
+                }
+                if (r + 1 < R) {  // x is in place and the accumulator read: the next reference's layer 1
+                    tc_fence_before();
+                    arrive_warp(&a_ready[s]);
+                }
+                uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};  // output layer on the BF16-rounded h3
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const ulonglong2 w = w4[j];
+                    const float2 u0 = unbf2(h3[2 * j]), u1 = unbf2(h3[2 * j + 1]);
+                    acc[2 * (j & 1)] = fma_pair(w.x, pair2(u0.x, u0.y), acc[2 * (j & 1)]);
+                    acc[2 * (j & 1) + 1] = fma_pair(w.y, pair2(u1.x, u1.y), acc[2 * (j & 1) + 1]);
+                }
+                const float2 s0 = unpair2(add_pair(add_pair(acc[0], acc[1]), add_pair(acc[2], acc[3])));
+                sum = s0.x + s0.y;
+                // the second half's sum meets the first half's here; it is rewritten only after the
+                // next reference's three layers, to which the first half contributes after reading it
+                if (h == 1) {
+                    part_s[s * 128 + i] = sum;
+                    arrive_warp(&part_ready[s]);
+                }
             }
+            if (!put_out(R - 1)) goto done;
         }
     }
 done:
     if (*abort_flag && threadIdx.x == 0) report(a.status, kDevTimeout);
     tc_fence_before();
     __syncthreads();
-    if (warp == 8) {
+    if (warp == kEpiWarps) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256u)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols)
                      : "memory");
     }
 }
