@@ -127,6 +127,72 @@ __global__ void __launch_bounds__(kPearsonThreads)
     }
 }
 
+// The same volume in one launch, for grids whose time is mostly launches and latency: every CTA
+// (two member halves x G vertex groups) gathers and centres the reference column itself, with the
+// first members' rows already in flight (32 per thread with one vertex each: below two waves of
+// CTAs the rows in flight per SM set the rate).  Per vertex the same sums in the same order as above, so
+// a grid's volume and its slabs' volumes are the same bits whichever kernel a size takes.
+template <int VEC, int G>
+__global__ void __launch_bounds__(2 * G)
+    pearson_small_kernel(const float* __restrict__ ref_field, int64_t N_ref, int64_t ref,
+                         const double* __restrict__ ref_mean, const double* __restrict__ s_ref_ptr,
+                         const float* __restrict__ field, int M, int64_t N, const double* __restrict__ mean,
+                         const double* __restrict__ inv_norm, float* __restrict__ out) {
+    using L = VecLoad<VEC>;
+    extern __shared__ float xs_all[];  // [M]
+    __shared__ float red[VEC * G];
+    const int g = threadIdx.x % G, half = threadIdx.x / G;
+    const int64_t v0 = ((int64_t)blockIdx.x * G + g) * VEC;
+    const bool active = v0 < N;
+    constexpr int B = VEC == 1 ? 32 : 8;  // rows in flight
+    const float* p = field + (int64_t)half * N + (active ? v0 : 0);
+    const int64_t step = 2 * N;
+    typename L::T y[B];
+#pragma unroll
+    for (int u = 0; u < B; ++u)
+        if (half + 2 * u < M) y[u] = L::ld(p + u * step);
+    const double mu_ref = ref_mean[ref];
+    for (int m = threadIdx.x; m < M; m += 2 * G) xs_all[m] = (float)((double)ref_field[m * N_ref + ref] - mu_ref);
+    float mu[VEC], acc[VEC];
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) {
+        mu[i] = active ? (float)mean[v0 + i] : 0.0f;
+        acc[i] = 0.0f;
+    }
+    __syncthreads();
+    for (int j = half; j < M; j += 2 * B) {
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            if (j + 2 * u >= M) break;
+            const float xm = xs_all[j + 2 * u];
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) acc[i] = fmaf(xm, L::get(y[u], i) - mu[i], acc[i]);
+        }
+        p += B * step;
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            if (j + 2 * B + 2 * u < M) y[u] = L::ld(p + u * step);
+    }
+    if (half == 1) {
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) red[i * G + g] = acc[i];
+    }
+    __syncthreads();
+    if (half == 0 && active) {
+        const double s_ref = *s_ref_ptr;
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            double a = (double)acc[i] + (double)red[i * G + g];
+            double r = a * s_ref * inv_norm[v0 + i];
+            r = r > 1.0 ? 1.0 : (r < -1.0 ? -1.0 : r);
+            out[v0 + i] = (float)r;
+        }
+    }
+}
+
+constexpr int64_t kPearsonOneMax = 65536, kPearsonFourMax = 262144;
+constexpr int64_t kPearsonSmallM = 8192;  // the reference column in 48 KB of shared memory
+
 cudaError_t launch_pearson(ndf_ctx* ctx, const Field& rf, const Field& qf, int64_t ref_idx,
                            float* out) {
     // the reference column comes from rf (N_ref vertices), the volume from qf (N vertices)
@@ -134,6 +200,22 @@ cudaError_t launch_pearson(ndf_ctx* ctx, const Field& rf, const Field& qf, int64
     const int64_t Mpad = (M + 3) & ~int64_t(3);
     cudaError_t e = ctx->stage_x.reserve(sizeof(float) * (size_t)Mpad);
     if (e != cudaSuccess) return e;
+    // Small grids in one launch.  Measured (us a volume, two launches / one): M = 100: 14.4 / 6.2
+    // at 1024 vertices, 14.4 / 7.3 at 20,000, 22.2 / 8.5 at 50,000, 24.2 / 14.4 at 120,000, 35.2 /
+    // 33.1 at 400,000; M = 1000: 51 / 23, 135 / 33, 137 / 42, 144 / 80, 236 / 245.  One vertex per
+    // thread up to kPearsonOneMax (137 / 75 us at 80,000, M = 1000, against 69 with four), four
+    // above; N % 4 != 0 above it stays with the two launches (75 against 83 us at 110,889), as
+    // does everything from kPearsonFourMax on, where the reference gather per CTA costs more
+    // than the launch.
+    if (M <= kPearsonSmallM && (N <= kPearsonOneMax || (N % 4 == 0 && N <= kPearsonFourMax))) {
+        const size_t sh = sizeof(float) * (size_t)M;
+        const int64_t per = N <= kPearsonOneMax ? 128 : 512;
+        auto kern = N <= kPearsonOneMax ? pearson_small_kernel<1, 128> : pearson_small_kernel<4, 128>;
+        kern<<<(unsigned)((N + per - 1) / per), 256, sh, ctx->stream>>>(
+            rf.data, N_ref, ref_idx, rf.mean, rf.inv_norm + ref_idx, qf.data, (int)M, N, qf.mean, qf.inv_norm, out);
+        ctx->launches++;
+        return cudaGetLastError();
+    }
     float* xt = ctx->stage_x.as<float>();
     unsigned* status = ctx->flag.as<unsigned>() + 1;
     int sb = (int)((Mpad + 255) / 256);
