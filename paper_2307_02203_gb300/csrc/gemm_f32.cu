@@ -184,22 +184,38 @@ __device__ __forceinline__ void for_results(const u64 (&acc)[8][4], int64_t m0, 
         }
 }
 
-// The tile's results row by row: f(row, column, v) for four consecutive columns, a warp covering
-// one row's 128 columns.  One copy of f in a loop: with f inlined once per result of a thread the
-// sine of the activations filled the instruction cache (26 us of a 43 us forward layer).
-template <class F>
-__device__ __forceinline__ void for_rows(Tile& S, const u64 (&acc)[8][4], int64_t m0, int64_t n0, F&& f) {
+// The tile's results row by row: f(row, column, v, e) for four consecutive columns, a warp covering
+// one row's 128 columns; e = fetch(row, column), read two iterations of the loop ahead of its use
+// (its latency cost 6 us of a 28 us backward layer).  Two copies of f in a loop: with f inlined
+// once per result of a thread the sine of the activations filled the instruction cache (26 us of
+// a 43 us forward layer).
+template <class Fetch, class F>
+__device__ __forceinline__ void for_rows(Tile& S, const u64 (&acc)[8][4], int64_t m0, int64_t n0, Fetch&& fetch,
+                                         F&& f) {
+    const int n = (threadIdx.x & 31) * 4;
+    int m = threadIdx.x >> 5;
+    float4 e[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) e[r] = fetch(m0 + m + 4 * r, n0 + n);
     __syncthreads();  // the operand slices are done with
-    for_results(acc, 0, 0, [&](int64_t m, int64_t n, float(&v)[4]) {
-        *reinterpret_cast<float4*>(&S.out[m][n]) = make_float4(v[0], v[1], v[2], v[3]);
+    for_results(acc, 0, 0, [&](int64_t mm, int64_t nn, float(&v)[4]) {
+        *reinterpret_cast<float4*>(&S.out[mm][nn]) = make_float4(v[0], v[1], v[2], v[3]);
     });
     __syncthreads();
-    const int n = (threadIdx.x & 31) * 4;
 #pragma unroll 1
-    for (int m = threadIdx.x >> 5; m < kBM; m += kThreads / 32) {
-        const float4 q = *reinterpret_cast<const float4*>(&S.out[m][n]);
-        float v[4] = {q.x, q.y, q.z, q.w};
-        f(m0 + m, n0 + n, v);
+    for (; m < kBM; m += 8) {
+        float4 next[2], q[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            next[r] = fetch(m0 + m + 8 + 4 * r, n0 + n);
+            q[r] = *reinterpret_cast<const float4*>(&S.out[m + 4 * r][n]);
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            float v[4] = {q[r].x, q[r].y, q[r].z, q[r].w};
+            f(m0 + m + 4 * r, n0 + n, v, e[r]);
+            e[r] = next[r];
+        }
     }
 }
 
@@ -228,11 +244,16 @@ __global__ void __launch_bounds__(kThreads, 2)
     float4 cs;
     tile_product<false, true>(S, X + row0 * L.cin, W, L.rows, L.cout, m0, n0, 0, L.cin, L.cin, L.cin, xvec, wvec,
                               acc, cs);
-    for_rows(S, acc, m0, n0, [&](int64_t m, int64_t n, float(&v)[4]) {
+    const int64_t nb = n0 + (threadIdx.x & 31) * 4;
+    float bn[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bn[j] = nb + j < L.cout ? bias[nb + j] : 0.0f;
+    auto nothing = [](int64_t, int64_t) { return make_float4(0.0f, 0.0f, 0.0f, 0.0f); };
+    for_rows(S, acc, m0, n0, nothing, [&](int64_t m, int64_t n, float(&v)[4], const float4&) {
         if (m >= L.rows || n >= L.cout) return;
         const int64_t left = L.cout - n, o = (row0 + m) * L.cout + n;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] += j < left ? bias[n + j] : 0.0f;
+        for (int j = 0; j < 4; ++j) v[j] += bn[j];
         store4(pre + o, v, left, yvec);
         if (post) {
 #pragma unroll
@@ -290,11 +311,15 @@ __global__ void __launch_bounds__(kThreads, 2) dense_backward_kernel(DenseLayer 
     const int64_t m0 = (int64_t)(tile / nt) * kBM, n0 = (int64_t)(tile % nt) * kBN;
     tile_product<false, false>(S, dY, L.W + z * L.wstride + a.col0, L.rows, dn, m0, n0, 0, L.cout, L.cout, L.cin,
                                a.yvec, a.wvec, acc, cs);
-    for_rows(S, acc, m0, n0, [&](int64_t m, int64_t n, float(&v)[4]) {
+    const int64_t m_end = min(m0 + kBM, L.rows);
+    auto fetch = [&](int64_t m, int64_t n) {
+        const int left = a.pre_in && m < m_end ? (int)min(dn - n, (int64_t)4) : 0;
+        return load4(a.pre_in + (row0 + m) * dn + n, left, a.dxvec);
+    };
+    for_rows(S, acc, m0, n0, fetch, [&](int64_t m, int64_t n, float(&v)[4], const float4& p) {
         if (m >= L.rows || n >= dn) return;
         const int64_t o = (row0 + m) * dn + n;
         if (a.pre_in) {
-            const float4 p = load4(a.pre_in + o, (int)min(dn - n, (int64_t)4), a.dxvec);
             v[0] *= dact_f(a.act, p.x);
             v[1] *= dact_f(a.act, p.y);
             v[2] *= dact_f(a.act, p.z);
