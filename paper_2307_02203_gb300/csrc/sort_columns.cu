@@ -60,40 +60,63 @@ __device__ __forceinline__ void sort_lane_registers(float (&a)[R]) {
     }
 }
 
+// a[r] *= s for every register, two per instruction (exact for s = +-1)
+template <int R>
+__device__ __forceinline__ void scale_registers(float (&a)[R], float s) {
+    if constexpr (R == 1) {
+        a[0] *= s;
+    } else {
+        const unsigned long long ss = ((unsigned long long)__float_as_uint(s) << 32) | __float_as_uint(s);
+#pragma unroll
+        for (int r = 0; r < R; r += 2) {
+            unsigned long long v = ((unsigned long long)__float_as_uint(a[r + 1]) << 32) | __float_as_uint(a[r]);
+            asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(v) : "l"(ss));
+            a[r] = __uint_as_float((unsigned)v);
+            a[r + 1] = __uint_as_float((unsigned)(v >> 32));
+        }
+    }
+}
+
 // the network on a warp's column in registers (element e = lane * R + r): each lane's
-// R registers sorted first, then the bitonic merges of runs R, 2R, .. 16R long
+// R registers sorted first, then the bitonic merges of runs R, 2R, .. 16R long.
+// In a stage across lanes the lower lane of a pair keeps the minimum and the upper one the
+// maximum.  Written as a choice that costs two ALU-pipe instructions per element, and the ALU
+// pipe bounds the sort; so the upper lanes of a stage hold their values negated: both lanes then
+// keep min(own, -received), and the sign changes from stage to stage are packed multiplications
+// by +-1 on the FMA pipe, which the sort leaves idle (352,000 columns of 1000 members from a
+// device-resident field: 1.96 -> 1.61 ms).
 template <int R>
 __device__ __forceinline__ void sort_warp_column(float (&a)[R]) {
     const int lane = threadIdx.x & 31;
+    float sign[5];  // by lane bit: -1 in the upper lanes
+#pragma unroll
+    for (int t = 0; t < 5; ++t) sign[t] = (lane >> t) & 1 ? -1.0f : 1.0f;
     sort_lane_registers<R>(a);
 #pragma unroll
-    for (int kk = 2 * R; kk <= 32 * R; kk <<= 1) {
-        // mirror stage: e and e ^ (kk - 1), across lanes since kk > R
+    for (int t = 0; t < 5; ++t) {  // merges of runs R << t
+        // mirror stage: e and e ^ (2R 2^t - 1): every lane bit up to t flipped, registers reversed
+        scale_registers<R>(a, sign[t]);
         {
-            const int lm = (kk - 1) / R;              // lane bits flipped
-            const bool lower = (lane & ((kk >> 1) / R)) == 0;
             float p[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) p[r] = __shfl_xor_sync(0xffffffffu, a[R - 1 - r], lm);
+            for (int r = 0; r < R; ++r) p[r] = __shfl_xor_sync(0xffffffffu, a[R - 1 - r], (2 << t) - 1);
 #pragma unroll
-            for (int r = 0; r < R; ++r) a[r] = lower ? fminf(a[r], p[r]) : fmaxf(a[r], p[r]);
+            for (int r = 0; r < R; ++r) a[r] = fminf(a[r], -p[r]);
         }
-        // half-cleaners: e and e ^ j
+        // half-cleaners: e and e ^ j, across lanes ..
 #pragma unroll
-        for (int j = kk >> 2; j > 0; j >>= 1) {
-            if (j < R) {
+        for (int u = t - 1; u >= 0; --u) {
+            scale_registers<R>(a, sign[u + 1] * sign[u]);
 #pragma unroll
-                for (int r = 0; r < R; ++r)
-                    if ((r & j) == 0) cmpx(a[r], a[r ^ j]);
-            } else {
-                const int lm = j / R;
-                const bool lower = (lane & lm) == 0;
+            for (int r = 0; r < R; ++r) a[r] = fminf(a[r], -__shfl_xor_sync(0xffffffffu, a[r], 1 << u));
+        }
+        scale_registers<R>(a, sign[0]);
+        // .. and inside a lane
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float q = __shfl_xor_sync(0xffffffffu, a[r], lm);
-                    a[r] = lower ? fminf(a[r], q) : fmaxf(a[r], q);
-                }
-            }
+        for (int j = R >> 1; j > 0; j >>= 1) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if ((r & j) == 0) cmpx(a[r], a[r ^ j]);
         }
     }
 }
