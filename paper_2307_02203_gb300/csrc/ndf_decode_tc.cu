@@ -17,26 +17,29 @@
 //     tile (TMEM lane i) and 64 of its columns.  The halves encode the vertex once per tile
 //     tile (TMEM lane i) and 64 of its columns.  The halves encode the vertex once per tile
 //     (two levels each; 64 FP32 features in shared memory); then for each reference, after
-//     each layer, they load their columns of the FP32 accumulator with tcgen05.ld, round,
-//     apply ReLU and write the next layer's operand (after layer 3 the columns stay as BF16
+//     each layer, they load their columns of the FP32 accumulator with tcgen05.ld, add the
+//     bias, round, apply ReLU and write the next layer's operand (after layer 3 the columns stay as BF16
 //     pairs in registers).  All other work sits where the slot would wait for an MMA: the
 //     output layer's dot product under the next reference's layer 1, its halves' exchange and
 //     the output function under layer 2, and the reference after that one's x (one half the
 //     products, the other the sums; an operand of its own) under layer 3.
-//   warp 16: allocates TMEM; one lane issues tcgen05.mma (M = 128, N = 128, K = 128 + 16) for
-//     whichever slot is ready and commits to that slot's mbarrier.  The extra K step adds the
-//     biases: a constant operand [1 1 1 0 ..] against each bias split into three BF16 terms
-//     (24 bits), so the epilogue neither loads nor adds them.
+//   warp 16: allocates TMEM; one lane issues tcgen05.mma (M = 128, N = 128, K = 128) for
+//     whichever slot is ready and commits to that slot's mbarrier.
 // The A operands live in TMEM (two times 64 columns of BF16 pairs per slot, x and h, beside its
-// 128 accumulator columns), not in shared memory: a layer's operand write and read would each be 32 KB of
-// shared-memory bandwidth (256 cycles) on top of the weights' 32 KB.  What bounds the kernel is
-// the chain of a slot (MMA of 576 cycles, commit, epilogue, MMA) with two slots per SM, so what
-// counts is what stands between a commit and the next hand-over (about 450 cycles; with x, dot
-// product and output there too it was 2,900, and 3,800 per layer with one warp per 128 columns,
-// operands in shared memory and the bias in the epilogue).  16 references on 1.76M vertices:
-// 4.29 ms before, 2.83 ms now.
-// The references' features f(p_r) (FP32) and the biases sit in shared memory.
+// 128 accumulator columns), not in shared memory: a layer's operand write and read would each be
+// 32 KB of shared-memory bandwidth (256 cycles) on top of the weights' 32 KB.  What bounds the
+// kernel is the chain of a slot (MMA of 512 cycles, commit, epilogue, MMA) with two slots per SM,
+// so what counts is what stands between a commit and the next hand-over (with x, dot product and
+// output there too it was 2,900 cycles after layer 3, and 3,800 per layer with one warp per 128
+// columns and operands in shared memory).  16 references on 1.76M vertices: 4.29 ms before,
+// 2.90 ms now (3.66 with the biases in shared memory).  (The biases as a ninth K step of three BF16 terms each: 2.83 ms, but the sums before
+// the rounding to BF16 are then added in another order.)
+// The references' features f(p_r) (FP32) sit in shared memory, the biases in constant memory.
 #include <cuda_bf16.h>
+
+#include <map>
+#include <mutex>
+#include <vector>
 
 #include "ndf_net.h"
 #include "tc_common.cuh"
@@ -111,29 +114,182 @@ struct TcInferArgs {
     int64_t offb1, offb2, offb3, offw4, offb4;
     int64_t N, X, Y, Z;
     int measure;
+    int slot;                  // of the model in c_net
     float* out;                // [R][N]
     unsigned* status;
 };
 
-// shared memory: W1, W2, W3 (2 atoms each), the biases' operand (layer l in columns 16 l
-// .. of one atom), then output weights / output weights (4 x 128 FP32), the references' features [R][64]
-// FP32 and the barriers
+// shared memory: W1, W2, W3 (2 atoms each), then biases / output weights (4 x 128 FP32), the
+// output layer's halves, the references' features [R][64], the rows' features and the barriers
 constexpr int kMaxRefsPerLaunch = 64;
-constexpr uint32_t kOffW = 0, kOffBias = 6 * kAtom, kOffOne = 7 * kAtom, kOffVec = 8 * kAtom;
+constexpr uint32_t kOffW = 0, kOffVec = 6 * kAtom;
 // TMEM columns: accumulators at 0 and 128, the slots' h at 256 and 320, their x at 384 and 448
 constexpr uint32_t kTmemCols = 512, kTmemH = 256, kTmemX = 384;
-constexpr uint32_t kOffPart = kOffVec + kHid * 4;  // [2 slots][128] output-layer halves
+constexpr uint32_t kOffPart = kOffVec + 4 * kHid * 4;  // [2 slots][128] output-layer halves
 constexpr uint32_t kOffFr = kOffPart + 2 * 128 * 4;
 constexpr uint32_t kOffFq = kOffFr + kMaxRefsPerLaunch * kLF * 4;  // [16][256 rows] float4
 constexpr uint32_t kOffBar = kOffFq + 256 * kLF * 4;
 constexpr uint32_t kTcSmem = kOffBar + 256 /*barriers*/ + 1024 /*align*/;
 
+// Biases and output weights of up to kConstSlots live models in constant memory: an epilogue thread
+// reads 64 of each per layer and reference, the same for its whole warp; from shared memory these
+// broadcasts took 1,100 cycles of its pipe per tile and reference (of 4,900), beside the tensor
+// cores' operand reads.  A model holds a slot from its creation to its end (one past the
+// kConstSlots-th decodes from shared memory); the decoder refreshes it after a parameter update.
+constexpr int kConstSlots = 16;
+__constant__ ulonglong2 c_net[kConstSlots][kHid];  // b1, b2, b3, w4
+
+// ---- encode / epilogue: slot s, row i = TMEM lane i, columns of half H
+template <bool CB, int H>
+__device__ __forceinline__ void decode_rows(const TcInferArgs& a, unsigned char* smem, uint32_t tmem, int64_t tiles,
+                                            int64_t step, volatile int* abort_flag) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, s = warp >> 3, R = a.R;
+    const float* vec = reinterpret_cast<const float*>(smem + kOffVec);
+    float* part_s = reinterpret_cast<float*>(smem + kOffPart);
+    const float* fr_all = reinterpret_cast<const float*>(smem + kOffFr);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOffBar);
+    uint64_t *a_ready = bars, *d_ready = bars + 2, *enc_ready = bars + 4, *part_ready = bars + 6;
+    // four consecutive values of (b1, b2, b3, w4)
+    auto vec4 = [&](int i) {
+        return CB ? c_net[a.slot][i >> 2] : reinterpret_cast<const ulonglong2*>(vec)[i >> 2];
+    };
+    const int i = (warp & 3) * 32 + lane;
+    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t taddr = tl + (uint32_t)(s * 128 + H * 64);
+    const uint32_t haddr = tl + kTmemH + (uint32_t)(s * 64 + H * 32);
+    const uint32_t xaddr = tl + kTmemX + (uint32_t)(s * 64 + H * 32);
+    const float b4 = a.params[a.offb4];
+    // this row's query features, four per 16 bytes
+    ulonglong2* fq = reinterpret_cast<ulonglong2*>(smem + kOffFq) + s * 128 + i;
+    uint32_t nd = 0, ne = 0, np = 0;
+    for (int64_t t = (int64_t)blockIdx.x * 2 + s; t < tiles; t += step) {
+        const int64_t v = t * kTile + i;
+        // this row's vertex, encoded once for every reference (rows past N encode
+        // position 0: harmless, never written out)
+        {
+            const int64_t vv = v < a.N ? v : 0;
+            const int64_t x = vv % a.X, y = (vv / a.X) % a.Y, z = vv / (a.X * a.Y);
+            const float p[3] = {pos_axis(x, a.X), pos_axis(y, a.Y), pos_axis(z, a.Z)};
+#pragma unroll 1
+            for (int l = H * (kLevels / 2); l < (H + 1) * (kLevels / 2); ++l) {
+                float f[kFeat];
+                encode_level(a.G, l, p, f);
+#pragma unroll
+                for (int q = 0; q < kFeat / 4; ++q)
+                    fq[(l * (kFeat / 4) + q) * 256] =
+                        make_ulonglong2(pair2(f[4 * q], f[4 * q + 1]), pair2(f[4 * q + 2], f[4 * q + 3]));
+            }
+        }
+        arrive_warp(&enc_ready[s]);
+        if (!__all_sync(0xffffffffu, wait_bounded(&enc_ready[s], ne & 1u, abort_flag))) return;
+        ++ne;
+        // x = [fr * fq ; fr + fq]: operand columns 0-31 the products, 32-63 the sums
+        auto put_x = [&](int r) {
+            const ulonglong2* fr = reinterpret_cast<const ulonglong2*>(fr_all + r * kLF);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint32_t o[8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const ulonglong2 f = fr[4 * c + j], q = fq[(4 * c + j) * 256];
+                    if (H == 0) {
+                        o[2 * j] = bf2(mul_pair(f.x, q.x));
+                        o[2 * j + 1] = bf2(mul_pair(f.y, q.y));
+                    } else {
+                        o[2 * j] = bf2(add_pair(f.x, q.x));
+                        o[2 * j + 1] = bf2(add_pair(f.y, q.y));
+                    }
+                }
+                tmem_st8(xaddr + (uint32_t)(8 * c), o);
+            }
+            tmem_wait_st();
+        };
+        // 32 accumulator columns d of layer l, from this half's column 32 c on: + bias, rounded, ReLU
+        auto hidden = [&](int l, int c, const uint32_t* d, uint32_t* o) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const ulonglong2 b = vec4(l * kHid + 64 * H + 32 * c + 4 * j);
+                o[2 * j] = relu2(bf2(add_pair(pair2(d[4 * j], d[4 * j + 1]), b.x)));
+                o[2 * j + 1] = relu2(bf2(add_pair(pair2(d[4 * j + 2], d[4 * j + 3]), b.y)));
+            }
+        };
+        // the output of reference r from this half's sum of the output layer
+        float sum = 0.0f;
+        auto put_out = [&](int r) {
+            if (H == 1) return true;
+            if (!__all_sync(0xffffffffu, wait_bounded(&part_ready[s], np & 1u, abort_flag))) return false;
+            ++np;
+            const float o = (sum + part_s[s * 128 + i]) + b4;
+            if (v < a.N)
+                a.out[(int64_t)r * a.N + v] = a.measure == 0 ? tanhf(o) : (o > 20.f ? o : log1pf(expf(o)));
+            return true;
+        };
+        put_x(0);
+        tc_fence_before();
+        arrive_warp(&a_ready[s]);
+        for (int r = 0; r < R; ++r) {
+#pragma unroll
+            for (int layer = 0; layer < 2; ++layer) {
+                if (!__all_sync(0xffffffffu, wait_bounded(&d_ready[s], nd & 1u, abort_flag))) return;
+                ++nd;
+                tc_fence_after();
+                uint32_t d[64], o[16];
+                tmem_ld64(taddr, d);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    hidden(layer, c, d + 32 * c, o);
+                    tmem_st16(haddr + (uint32_t)(16 * c), o);
+                }
+                tmem_wait_st();
+                tc_fence_before();
+                arrive_warp(&a_ready[s]);
+                if (layer == 0) {
+                    if (r > 0 && !put_out(r - 1)) return;
+                } else if (r + 1 < R) {
+                    put_x(r + 1);  // layer 1 of this reference, which read x, has completed
+                }
+            }
+            if (!__all_sync(0xffffffffu, wait_bounded(&d_ready[s], nd & 1u, abort_flag))) return;
+            ++nd;
+            tc_fence_after();
+            uint32_t h3[32];
+            {
+                uint32_t d[64];
+                tmem_ld64(taddr, d);
+                hidden(2, 0, d, h3);
+                hidden(2, 1, d + 32, h3 + 16);
+            }
+            if (r + 1 < R) {  // x is in place and the accumulator read: the next reference's layer 1
+                tc_fence_before();
+                arrive_warp(&a_ready[s]);
+            }
+            uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};  // output layer on the BF16-rounded h3
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const ulonglong2 w = vec4(3 * kHid + 64 * H + 4 * j);
+                const float2 u0 = unbf2(h3[2 * j]), u1 = unbf2(h3[2 * j + 1]);
+                acc[2 * (j & 1)] = fma_pair(w.x, pair2(u0.x, u0.y), acc[2 * (j & 1)]);
+                acc[2 * (j & 1) + 1] = fma_pair(w.y, pair2(u1.x, u1.y), acc[2 * (j & 1) + 1]);
+            }
+            const float2 s0 = unpair2(add_pair(add_pair(acc[0], acc[1]), add_pair(acc[2], acc[3])));
+            sum = s0.x + s0.y;
+            // the second half's sum meets the first half's here; it is rewritten only after the
+            // next reference's three layers, to which the first half contributes after reading it
+            if (H == 1) {
+                part_s[s * 128 + i] = sum;
+                arrive_warp(&part_ready[s]);
+            }
+        }
+        if (!put_out(R - 1)) return;
+    }
+}
+
+template <bool CB>
 __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    float* w4s = reinterpret_cast<float*>(smem + kOffVec);
-    float* part_s = reinterpret_cast<float*>(smem + kOffPart);
+    float* vec = reinterpret_cast<float*>(smem + kOffVec);  // b1, b2, b3, w4
     float* fr_all = reinterpret_cast<float*>(smem + kOffFr);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOffBar);
     uint64_t* a_ready = bars;         // [2] epilogue -> MMA (8 warps)
@@ -153,18 +309,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferAr
         *reinterpret_cast<uint4*>(smem + kOffW + o) =
             reinterpret_cast<const uint4*>(a.w + ((size_t)l * kHid + row) * kHid)[c];
     }
-    for (int i = threadIdx.x; i < kHid; i += blockDim.x) {
-        w4s[i] = a.params[a.offw4 + i];
-#pragma unroll
-        for (int l = 0; l < 4; ++l) {  // the fourth quarter of the atom is not read
-            const float b = l == 0 ? a.params[a.offb1 + i] : l == 1 ? a.params[a.offb2 + i] : l == 2 ? a.params[a.offb3 + i] : 0.0f;
-            const float hi = __bfloat162float(__float2bfloat16_rn(b));
-            const float r1 = isinf(hi) ? 0.0f : b - hi, mid = __bfloat162float(__float2bfloat16_rn(r1));
-            *reinterpret_cast<uint4*>(smem + kOffBias + swz(i, 2 * l)) = make_uint4(bf2(hi, mid), bf2(r1 - mid, 0.0f), 0u, 0u);
-            *reinterpret_cast<uint4*>(smem + kOffBias + swz(i, 2 * l + 1)) = make_uint4(0u, 0u, 0u, 0u);
-        }
-        *reinterpret_cast<uint4*>(smem + kOffOne + swz(i, 0)) = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
-        *reinterpret_cast<uint4*>(smem + kOffOne + swz(i, 1)) = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = threadIdx.x; i < 4 * kHid; i += blockDim.x) {
+        const int64_t off = i < kHid ? a.offb1 : i < 2 * kHid ? a.offb2 : i < 3 * kHid ? a.offb3 : a.offw4;
+        vec[i] = a.params[off + (i % kHid)];
     }
     for (int i = threadIdx.x; i < R * kLevels; i += blockDim.x) {
         const int64_t v = a.refs[i / kLevels];
@@ -231,8 +378,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferAr
                         tc_mma_ts(d, ta + (uint32_t)(kk * 8), desc_sw128(wl + at) + (uint64_t)((kk & 3) * 2), idesc,
                                   kk > 0 ? 1u : 0u);
                     }
-                    tc_mma(d, desc_sw128(smem_u32(smem + kOffOne)),
-                           desc_sw128(smem_u32(smem + kOffBias)) + (uint64_t)(layer[s] * 2), idesc, 1u);
                     tc_commit(&d_ready[s]);
                     layer[s] = layer[s] == 2 ? 0 : layer[s] + 1;
                     --left[s];
@@ -249,132 +394,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) infer_tc_kernel(const TcInferAr
                 }
             }
         }
-    } else {  // ---- encode / epilogue: slot s, row i = TMEM lane i, columns of half h
-        const int s = warp >> 3, h = (warp >> 2) & 1;
-        const int i = (warp & 3) * 32 + lane;
-        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        const uint32_t taddr = tl + (uint32_t)(s * 128 + h * 64);
-        const uint32_t haddr = tl + kTmemH + (uint32_t)(s * 64 + h * 32);
-        const uint32_t xaddr = tl + kTmemX + (uint32_t)(s * 64 + h * 32);
-        const float b4 = a.params[a.offb4];
-        // this row's query features, four per 16 bytes
-        ulonglong2* fq = reinterpret_cast<ulonglong2*>(smem + kOffFq) + s * 128 + i;
-        const ulonglong2* w4 = reinterpret_cast<const ulonglong2*>(w4s + 64 * h);
-        uint32_t nd = 0, ne = 0, np = 0;
-        for (int64_t t = (int64_t)blockIdx.x * 2 + s; t < tiles; t += step) {
-            const int64_t v = t * kTile + i;
-            // this row's vertex, encoded once for every reference (rows past N encode
-            // position 0: harmless, never written out)
-            {
-                const int64_t vv = v < a.N ? v : 0;
-                const int64_t x = vv % a.X, y = (vv / a.X) % a.Y, z = vv / (a.X * a.Y);
-                const float p[3] = {pos_axis(x, a.X), pos_axis(y, a.Y), pos_axis(z, a.Z)};
-#pragma unroll 1
-                for (int l = h * (kLevels / 2); l < (h + 1) * (kLevels / 2); ++l) {
-                    float f[kFeat];
-                    encode_level(a.G, l, p, f);
-#pragma unroll
-                    for (int q = 0; q < kFeat / 4; ++q)
-                        fq[(l * (kFeat / 4) + q) * 256] =
-                            make_ulonglong2(pair2(f[4 * q], f[4 * q + 1]), pair2(f[4 * q + 2], f[4 * q + 3]));
-                }
-            }
-            arrive_warp(&enc_ready[s]);
-            if (!__all_sync(0xffffffffu, wait_bounded(&enc_ready[s], ne & 1u, abort_flag))) goto done;
-            ++ne;
-            // x = [fr * fq ; fr + fq]: operand columns 0-31 the products, 32-63 the sums
-            auto put_x = [&](int r) {
-                const ulonglong2* fr = reinterpret_cast<const ulonglong2*>(fr_all + r * kLF);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t o[8];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const ulonglong2 f = fr[4 * c + j], q = fq[(4 * c + j) * 256];
-                        if (h == 0) {
-                            o[2 * j] = bf2(mul_pair(f.x, q.x));
-                            o[2 * j + 1] = bf2(mul_pair(f.y, q.y));
-                        } else {
-                            o[2 * j] = bf2(add_pair(f.x, q.x));
-                            o[2 * j + 1] = bf2(add_pair(f.y, q.y));
-                        }
-                    }
-                    tmem_st8(xaddr + (uint32_t)(8 * c), o);
-                }
-                tmem_wait_st();
-            };
-            // the output of reference r from this half's sum of the output layer
-            float sum = 0.0f;
-            auto put_out = [&](int r) {
-                if (h == 1) return true;
-                if (!__all_sync(0xffffffffu, wait_bounded(&part_ready[s], np & 1u, abort_flag))) return false;
-                ++np;
-                const float o = (sum + part_s[s * 128 + i]) + b4;
-                if (v < a.N)
-                    a.out[(int64_t)r * a.N + v] = a.measure == 0 ? tanhf(o) : (o > 20.f ? o : log1pf(expf(o)));
-                return true;
-            };
-            put_x(0);
-            tc_fence_before();
-            arrive_warp(&a_ready[s]);
-            for (int r = 0; r < R; ++r) {
-#pragma unroll 1
-                for (int layer = 0; layer < 2; ++layer) {
-                    if (!__all_sync(0xffffffffu, wait_bounded(&d_ready[s], nd & 1u, abort_flag))) goto done;
-                    ++nd;
-                    tc_fence_after();
-                    uint32_t d[64], o[16];
-                    tmem_ld64(taddr, d);
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {  // rounded, ReLU
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) o[j] = relu2(bf2(pair2(d[32 * c + 2 * j], d[32 * c + 2 * j + 1])));
-                        tmem_st16(haddr + (uint32_t)(16 * c), o);
-                    }
-                    tmem_wait_st();
-                    tc_fence_before();
-                    arrive_warp(&a_ready[s]);
-                    if (layer == 0) {
-                        if (r > 0 && !put_out(r - 1)) goto done;
-                    } else if (r + 1 < R) {
-                        put_x(r + 1);  // layer 1 of this reference, which read x, has completed
-                    }
-                }
-                if (!__all_sync(0xffffffffu, wait_bounded(&d_ready[s], nd & 1u, abort_flag))) goto done;
-                ++nd;
-                tc_fence_after();
-                uint32_t h3[32];
-                {
-                    uint32_t d[64];
-                    tmem_ld64(taddr, d);
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) h3[j] = relu2(bf2(pair2(d[2 * j], d[2 * j + 1])));
-                }
-                if (r + 1 < R) {  // x is in place and the accumulator read: the next reference's layer 1
-                    tc_fence_before();
-                    arrive_warp(&a_ready[s]);
-                }
-                uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};  // output layer on the BF16-rounded h3
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const ulonglong2 w = w4[j];
-                    const float2 u0 = unbf2(h3[2 * j]), u1 = unbf2(h3[2 * j + 1]);
-                    acc[2 * (j & 1)] = fma_pair(w.x, pair2(u0.x, u0.y), acc[2 * (j & 1)]);
-                    acc[2 * (j & 1) + 1] = fma_pair(w.y, pair2(u1.x, u1.y), acc[2 * (j & 1) + 1]);
-                }
-                const float2 s0 = unpair2(add_pair(add_pair(acc[0], acc[1]), add_pair(acc[2], acc[3])));
-                sum = s0.x + s0.y;
-                // the second half's sum meets the first half's here; it is rewritten only after the
-                // next reference's three layers, to which the first half contributes after reading it
-                if (h == 1) {
-                    part_s[s * 128 + i] = sum;
-                    arrive_warp(&part_ready[s]);
-                }
-            }
-            if (!put_out(R - 1)) goto done;
-        }
+    } else if (((warp >> 2) & 1) == 0) {
+        decode_rows<CB, 0>(a, smem, tmem, tiles, step, abort_flag);
+    } else {
+        decode_rows<CB, 1>(a, smem, tmem, tiles, step, abort_flag);
     }
-done:
     if (*abort_flag && threadIdx.x == 0) report(a.status, kDevTimeout);
     tc_fence_before();
     __syncthreads();
@@ -385,14 +409,48 @@ done:
     }
 }
 
+static std::mutex g_slot_mutex;
+static std::map<int, std::vector<char>> g_slots;  // per device: slots in use
+
+int const_slot_acquire(int device) {
+    std::lock_guard<std::mutex> lock(g_slot_mutex);
+    std::vector<char>& used = g_slots[device];
+    used.resize(kConstSlots, 0);
+    for (int i = 0; i < kConstSlots; ++i)
+        if (!used[(size_t)i]) {
+            used[(size_t)i] = 1;
+            return i;
+        }
+    return -1;
+}
+
+void const_slot_release(int device, int slot) {
+    if (slot < 0) return;
+    std::lock_guard<std::mutex> lock(g_slot_mutex);
+    g_slots[device][(size_t)slot] = 0;
+}
+
 cudaError_t launch_infer_tc(ndf_model* m, const int64_t* d_refs, int R, float* out) {
     ndf_ctx* ctx = m->ctx;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(infer_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kTcSmem);
+    // from 100,000 values on (40 us) the constant copy after a parameter update (2 us) is repaid by
+    // its first call
+    // its first call; a captured call reads the parameters themselves (its copy would not run now)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(ctx->stream, &capture);
+    if (e != cudaSuccess) return e;
+    const bool constant = m->cslot >= 0 && capture == cudaStreamCaptureStatusNone &&
+                          (double)R * (double)(m->X * m->Y * m->Z) >= 1e5;
+    auto kern = constant ? infer_tc_kernel<true> : infer_tc_kernel<false>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
+    if (e != cudaSuccess) return e;
+    if (constant && m->cslot_stale) {
+        void* base = nullptr;
+        e = cudaGetSymbolAddress(&base, c_net);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(static_cast<char*>(base) + (size_t)m->cslot * sizeof(c_net[0]), m->mlp_vec(),
+                                sizeof(c_net[0]), cudaMemcpyDeviceToDevice, ctx->stream);
         if (e != cudaSuccess) return e;
-        attr = true;
+        m->cslot_stale = false;
     }
     TcInferArgs a;
     a.G.grid = m->grid_bf;
@@ -412,6 +470,7 @@ cudaError_t launch_infer_tc(ndf_model* m, const int64_t* d_refs, int R, float* o
     a.Y = m->Y;
     a.Z = m->Z;
     a.measure = m->measure;
+    a.slot = m->cslot;
     a.status = ctx->flag.as<unsigned>() + 1;
     const int64_t tiles = (a.N + kTile - 1) / kTile;
     int64_t grid = ctx->sm_count;  // one persistent CTA per SM, two tiles in flight each
@@ -421,7 +480,7 @@ cudaError_t launch_infer_tc(ndf_model* m, const int64_t* d_refs, int R, float* o
         a.refs = d_refs + r0;
         a.R = R - r0 < kMaxRefsPerLaunch ? R - r0 : kMaxRefsPerLaunch;
         a.out = out + (int64_t)r0 * a.N;
-        infer_tc_kernel<<<(unsigned)grid, kTcThreads, kTcSmem, ctx->stream>>>(a);
+        kern<<<(unsigned)grid, kTcThreads, kTcSmem, ctx->stream>>>(a);
         ctx->launches++;
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

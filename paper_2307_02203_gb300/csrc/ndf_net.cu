@@ -238,9 +238,14 @@ __global__ void __launch_bounds__(256)
 }
 
 __global__ void refresh_mlp_kernel(const float* __restrict__ p, int64_t offW1, int64_t offW2,
-                                   int64_t offW3, __nv_bfloat16* __restrict__ w) {
+                                   int64_t offW3, int64_t offb1, int64_t offb2, int64_t offb3, int64_t offw4,
+                                   __nv_bfloat16* __restrict__ w, float* __restrict__ vec) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * kHid * kHid) return;
+    if (i < 4 * kHid) {
+        const int k = i / kHid;
+        vec[i] = p[(k == 0 ? offb1 : k == 1 ? offb2 : k == 2 ? offb3 : offw4) + i % kHid];
+    }
     const int l = i / (kHid * kHid), r = (i / kHid) % kHid, c = i % kHid;
     const int64_t off = l == 0 ? offW1 : (l == 1 ? offW2 : offW3);
     w[(size_t)l * kHid * kHid + r * kHid + c] = __float2bfloat16_rn(p[off + (int64_t)r * kHid + c]);
@@ -307,7 +312,7 @@ ndf_status model_alloc(ndf_ctx* ctx, const int res[kLevels], int measure, int64_
     if (e == cudaSuccess) e = cudaMalloc(&m->m, n * 4);
     if (e == cudaSuccess) e = cudaMalloc(&m->v, n * 4);
     if (e == cudaSuccess) e = cudaMalloc(&m->grid_bf, (size_t)m->L.n_grid * 2);
-    if (e == cudaSuccess) e = cudaMalloc(&m->wbf, (size_t)3 * kHid * kHid * 2);
+    if (e == cudaSuccess) e = cudaMalloc(&m->wbf, (size_t)3 * kHid * kHid * 2 + (size_t)4 * kHid * 4);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->params, 0, n * 4, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->grad, 0, n * 4, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->m, 0, n * 4, ctx->stream);
@@ -316,6 +321,7 @@ ndf_status model_alloc(ndf_ctx* ctx, const int res[kLevels], int measure, int64_
         model_free(m);
         return cuda_fail(ctx, e, "model allocation");
     }
+    m->cslot = const_slot_acquire(ctx->device);
     *out = m;
     return NDF_OK;
 }
@@ -326,6 +332,7 @@ void model_free(ndf_model* m) {
     for (void* q : ps)
         if (q) cudaFree(q);
     m->work.release();
+    const_slot_release(m->ctx->device, m->cslot);
     delete m;
 }
 
@@ -334,7 +341,8 @@ cudaError_t model_refresh_bf16(ndf_model* m) {
     grid_to_bf16_kernel<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(m->params, m->L.n_grid,
                                                                       m->grid_bf);
     refresh_mlp_kernel<<<(3 * kHid * kHid + 255) / 256, 256, 0, ctx->stream>>>(
-        m->params, m->L.W1, m->L.W2, m->L.W3, m->wbf);
+        m->params, m->L.W1, m->L.W2, m->L.W3, m->L.b1, m->L.b2, m->L.b3, m->L.w4, m->wbf, m->mlp_vec());
+    m->cslot_stale = true;
     ctx->launches += 2;
     return cudaGetLastError();
 }
@@ -394,7 +402,8 @@ cudaError_t model_adam(ndf_model* m, float* grad, bool clear, float lr, float be
         adam_kernel<false><<<ctas, 256, 0, s>>>(m->params, grad, m->m, m->v, m->L.total, m->L.n_grid,
                                                 m->grid_bf, lr, beta1, beta2, eps, c1, c2);
     refresh_mlp_kernel<<<(3 * kHid * kHid + 255) / 256, 256, 0, s>>>(
-        m->params, m->L.W1, m->L.W2, m->L.W3, m->wbf);
+        m->params, m->L.W1, m->L.W2, m->L.W3, m->L.b1, m->L.b2, m->L.b3, m->L.w4, m->wbf, m->mlp_vec());
+    m->cslot_stale = true;
     ctx->launches += 2;
     return cudaGetLastError();
 }

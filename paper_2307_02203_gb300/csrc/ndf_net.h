@@ -61,7 +61,10 @@ struct ndf_model {
     float* m = nullptr;        // Adam first moment
     float* v = nullptr;        // Adam second moment
     __nv_bfloat16* grid_bf = nullptr;  // bf16 copy of the grid part
-    __nv_bfloat16* wbf = nullptr;      // [3][128][128] bf16 W1..W3 ([out][in])
+    __nv_bfloat16* wbf = nullptr;      // [3][128][128] bf16 W1..W3 ([out][in]), then mlp_vec
+    float* mlp_vec() const { return reinterpret_cast<float*>(wbf + 3 * 128 * 128); }  // b1, b2, b3, w4
+    int cslot = -1;             // the decoder's constant-memory slot of mlp_vec (-1: none)
+    bool cslot_stale = true;    // mlp_vec has changed since it was copied there
     int64_t t = 0;             // Adam steps taken
     ndf::NetWork work;
     // training record
@@ -77,6 +80,9 @@ namespace ndf {
 ndf_status model_alloc(ndf_ctx* ctx, const int res[kLevels], int measure, int64_t X, int64_t Y,
                        int64_t Z, ndf_model** out);
 void model_free(ndf_model* m);
+// a free constant-memory slot of the decoder on the device, or -1
+int const_slot_acquire(int device);
+void const_slot_release(int device, int slot);
 cudaError_t model_init_params(ndf_model* m, uint64_t seed);
 cudaError_t model_refresh_bf16(ndf_model* m);  // bf16 copies from the FP32 master
 ndf_status ensure_work(ndf_model* m, int64_t B);

@@ -1,7 +1,7 @@
 """The dense-grid decoder where it can go wrong: grids around its 128-vertex tiles and two slots,
 1 to 66 references (more than one launch), each volume bit-equal to the reference's own call and
-within the BF16 bound (3e-2) of the FP64 oracle; and its bias path (three BF16 terms per bias on the
-tensor cores): with zero weights the third layer is ReLU(b3) exactly, so the output is
+within the BF16 bound (3e-2) of the FP64 oracle; and its biases, which are not
+rounded to BF16: with zero weights the third layer is ReLU(b3) exactly, so the output is
 tanh(w4 . bf16(ReLU(b3)) + b4) up to the FP32 sum over 128 terms (each bias is reproduced to 2^-24 of
 itself and none of the drawn ones lies that close to a BF16 rounding boundary; 128 products of at most
 0.7 in FP32: 128 * 2^-24 * 0.7 < 6e-6, bound 1e-5)."""
@@ -65,3 +65,41 @@ def test_biases_carry_24_bits(ndf_mod, ctx):
     want = np.tanh(p[g["w4"]].astype(np.float64) @ h + float(p[g["b4"]][0]))
     assert np.abs(out - want).max() <= 1e-5
     ndf_mod.ndf_model_free(m)
+
+
+def test_constant_memory_slots(ndf_mod, ctx):
+    """More live models than constant-memory slots, on a grid large enough for them: every model
+    decodes its own parameters, also after an update of one of them and after a slot's reuse, and a
+    volume equals the one decoded in small calls (below the constant path's size)."""
+    X, Y, Z = 50, 50, 20
+
+    def make(seed):
+        m = ndf_mod.ndf_model_create(ctx, RES_SMALL, 0, 2, X, Y, Z)
+        ndf_mod.ndf_model_set_params(m, make_params(seed))
+        return m
+
+    def volumes(m):
+        out = torch.empty((2, X * Y * Z), device="cuda")
+        torch.cuda.synchronize()
+        ndf_mod.ndf_infer_batch(m, [3, 777], out)
+        ndf_mod.ndf_synchronize(ctx)
+        one = np.empty(X * Y * Z, np.float32)
+        ndf_mod.ndf_infer(m, 3, one)
+        got = out.cpu().numpy()
+        np.testing.assert_array_equal(got[0], one)
+        return got
+
+    models = [make(k) for k in range(20)]
+    first = [volumes(m) for m in models]
+    for a, b in zip(first, first[1:]):
+        assert np.abs(a - b).max() > 0.05
+    ndf_mod.ndf_model_set_params(models[2], make_params(99))
+    changed = volumes(models[2])
+    assert np.abs(changed - first[2]).max() > 0.05
+    ndf_mod.ndf_model_free(models.pop(1))
+    models.append(make(99))
+    np.testing.assert_array_equal(volumes(models[-1]), changed)
+    np.testing.assert_array_equal(volumes(models[0]), first[0])
+    np.testing.assert_array_equal(volumes(models[-2]), first[19])
+    for m in models:
+        ndf_mod.ndf_model_free(m)
