@@ -7,6 +7,32 @@
 
 namespace ndf {
 
+// Programmatic dependent launch.  A kernel that begins with pdl_wait() may be launched by
+// launch_after() while its predecessor on the stream still runs: its CTAs take the places that
+// the predecessor's leave, and pdl_wait() holds them until that grid has completed and its writes
+// are visible.  pdl_launch() in the predecessor allows it as soon as all its CTAs have started
+// (without it, when they have ended).  Hides the launch and the ramp of short dependent kernels.
+// Such a kernel takes what its predecessor writes through plain pointers: a load through a const
+// __restrict__ one (or __ldg) counts as invariant, and the compiler may move it above the wait.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+
 // Bit flags of the device status word (ctx->flag, word 1).
 enum : unsigned { kDevTimeout = 1u, kDevBadInput = 2u };
 

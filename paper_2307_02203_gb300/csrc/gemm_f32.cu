@@ -21,6 +21,7 @@
 //     summation: rounding grows with 16 + K / 16 terms instead of K).
 #include "gemm_f32.h"
 
+#include "device_common.cuh"
 #include "hash_common.cuh"
 
 namespace ndf {
@@ -58,7 +59,7 @@ __device__ __forceinline__ u64 twice(float a) {
 
 // four consecutive values p[0..3], the first n of them inside the matrix (vec: p is 16-byte
 // aligned whenever n >= 4)
-__device__ __forceinline__ float4 load4(const float* __restrict__ p, int n, bool vec) {
+__device__ __forceinline__ float4 load4(const float* p, int n, bool vec) {
     if (n >= 4 && vec) return *reinterpret_cast<const float4*>(p);
     float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (n > 0) v.x = p[0];
@@ -77,7 +78,7 @@ __device__ __forceinline__ int tile_tx() { return (threadIdx.x >> 6) * 8 + (thre
 // [N][K] (else [K][N]).  With TA csum = this thread's sums of A over its rows k (every 8th),
 // columns m0 + 4 (tid & 15) + 0 .. 3.
 template <bool TA, bool TB>
-__device__ __forceinline__ void tile_product(Tile& S, const float* __restrict__ A, const float* __restrict__ B,
+__device__ __forceinline__ void tile_product(Tile& S, const float* A, const float* B,
                                              int64_t M, int64_t N, int64_t m0, int64_t n0, int64_t k0,
                                              int64_t k1, int64_t lda, int64_t ldb, bool avec, bool bvec,
                                              u64 (&acc)[8][4], float4& csum) {
@@ -220,7 +221,7 @@ __device__ __forceinline__ void for_rows(Tile& S, const u64 (&acc)[8][4], int64_
 }
 
 // stores v[0..3] at p, the first n of them inside the matrix (vec as in load4)
-__device__ __forceinline__ void store4(float* __restrict__ p, const float (&v)[4], int64_t n, bool vec) {
+__device__ __forceinline__ void store4(float* p, const float (&v)[4], int64_t n, bool vec) {
     if (n >= 4 && vec) {
         *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
     } else {
@@ -232,9 +233,11 @@ __device__ __forceinline__ void store4(float* __restrict__ p, const float (&v)[4
 
 // grid: (row tiles x column tiles, 1, batch)
 __global__ void __launch_bounds__(kThreads, 2)
-    dense_forward_kernel(DenseLayer L, const float* __restrict__ X, float* __restrict__ pre,
-                         float* __restrict__ post, int act, bool xvec, bool wvec, bool yvec) {
+    dense_forward_kernel(DenseLayer L, const float* X, float* pre,
+                         float* post, int act, bool xvec, bool wvec, bool yvec) {
     __shared__ __align__(16) Tile S;
+    pdl_launch();
+    pdl_wait();
     const int nt = (L.cout + kBN - 1) / kBN, z = blockIdx.z;
     const int64_t m0 = (int64_t)(blockIdx.x / nt) * kBM, n0 = (int64_t)(blockIdx.x % nt) * kBN;
     const int64_t row0 = (int64_t)z * L.rows;
@@ -275,6 +278,8 @@ struct BackwardArgs {
 // grid: (weight-gradient tiles x splits, then data-gradient tiles; 1; batch)
 __global__ void __launch_bounds__(kThreads, 2) dense_backward_kernel(DenseLayer L, BackwardArgs a) {
     __shared__ __align__(16) Tile S;
+    pdl_launch();
+    pdl_wait();
     const int z = blockIdx.z;
     const int64_t row0 = (int64_t)z * L.rows;
     const float* dY = a.dY + row0 * L.cout;
@@ -339,6 +344,8 @@ struct GradSegs {
 // lanes' sums are added in order.  blockIdx.y: segment
 __global__ void __launch_bounds__(256) grad_sums_kernel(GradSegs g) {
     __shared__ float red[8][32];
+    pdl_launch();
+    pdl_wait();
     const GradSeg s = g.s[blockIdx.y];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     for (int64_t i0 = (int64_t)blockIdx.x * 32; i0 < s.n; i0 += (int64_t)gridDim.x * 32) {
@@ -370,9 +377,8 @@ cudaError_t dense_forward(cudaStream_t s, const DenseLayer& L, const float* X, f
     const int64_t tiles = (L.rows + kBM - 1) / kBM * ((L.cout + kBN - 1) / kBN);
     const bool wv = aligned16(L.W, L.cin) && (L.wstride & 3) == 0;
     const bool yv = aligned16(pre, L.cout) && (!post || aligned16(post, L.cout));
-    dense_forward_kernel<<<dim3((unsigned)tiles, 1, (unsigned)L.batch), kThreads, 0, s>>>(
-        L, X, pre, post, act, aligned16(X, L.cin), wv, yv);
-    return cudaGetLastError();
+    return launch_after(dense_forward_kernel, dim3((unsigned)tiles, 1, (unsigned)L.batch), dim3(kThreads), 0, s, L, X,
+                        pre, post, act, aligned16(X, L.cin), wv, yv);
 }
 
 int64_t dense_grad_floats(int64_t cin, int64_t cout) {
@@ -390,11 +396,11 @@ cudaError_t grad_sums_flush(cudaStream_t s, GradSums& g, uint64_t* launches) {
     k.count = g.count;
     int64_t bx = (nmax + 31) / 32;
     if (bx > 4096) bx = 4096;
-    grad_sums_kernel<<<dim3((unsigned)bx, (unsigned)g.count), 256, 0, s>>>(k);
     ++*launches;
+    const dim3 grid((unsigned)bx, (unsigned)g.count);
     g.count = 0;
     g.used = 0;
-    return cudaGetLastError();
+    return launch_after(grad_sums_kernel, grid, dim3(256), 0, s, k);
 }
 
 cudaError_t dense_backward(cudaStream_t s, const DenseLayer& L, const float* X, const float* dY, float* dX,
@@ -432,9 +438,9 @@ cudaError_t dense_backward(cudaStream_t s, const DenseLayer& L, const float* X, 
     a.yvec = aligned16(dY, L.cout);
     a.wvec = aligned16(L.W + col0, L.cin) && (L.wstride & 3) == 0;
     a.dxvec = dX && aligned16(dX, dn) && (!pre_in || aligned16(pre_in, dn));
-    dense_backward_kernel<<<dim3(a.wblocks + a.dblocks, 1, (unsigned)L.batch), kThreads, 0, s>>>(L, a);
     ++*launches;
-    return cudaGetLastError();
+    return launch_after(dense_backward_kernel, dim3(a.wblocks + a.dblocks, 1, (unsigned)L.batch), dim3(kThreads), 0, s,
+                        L, a);
 }
 
 }  // namespace ndf

@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(1024)
                      const int64_t* __restrict__ refs, int64_t ref0, float* __restrict__ xs_all,
                      int* __restrict__ perm_all, unsigned* __restrict__ status,
                      unsigned long long* __restrict__ work) {
+    pdl_launch();
     if (blockIdx.x == 0 && threadIdx.x == 0) *work = 0ull;  // the searches' work counter
     __shared__ float key[kKsgMaxM];
     __shared__ int val[kKsgMaxM];
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(128)
                           unsigned* __restrict__ status, unsigned long long* __restrict__ work) {
     const int lane = threadIdx.x & 31;
     const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    pdl_launch();
     if (row == 0 && lane == 0) *work = 0ull;
     if (row >= R) return;
     const int64_t ref = refs ? refs[row] : ref0 + row;
@@ -1039,6 +1041,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
     constexpr int KK = K1 - 1;
     constexpr int GT = 32 * kGroupWarps;
     constexpr unsigned FULL = 0xffffffffu;
+    pdl_wait();  // the staged references and the work counter
     extern __shared__ __align__(16) unsigned char smem[];
     const int M = A.M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int group = warp / kGroupWarps, gw = warp % kGroupWarps, gt = threadIdx.x % GT;
@@ -1372,10 +1375,10 @@ static cudaError_t launch_ksg_k(ndf_ctx* ctx, KsgArgs A, bool prune) {
             if (e != cudaSuccess) return e;
             int64_t grid = (int64_t)ctx->sm_count;
             if (grid * gpc > pairs) grid = (pairs + gpc - 1) / gpc;
-            kern<<<(unsigned)grid, threads, smem, ctx->stream>>>(A, ctx->ksg_work.as<unsigned long long>(), lw,
-                                                                 ctx->ksg_switch_min, ctx->ksg_every);
+            e = launch_after(kern, dim3((unsigned)grid), dim3((unsigned)threads), smem, ctx->stream, A,
+                             ctx->ksg_work.as<unsigned long long>(), lw, ctx->ksg_switch_min, ctx->ksg_every);
             ctx->launches++;
-            return cudaGetLastError();
+            return e;
         }
     }
     if (prune && ctx->ksg_algorithm == NDF_KSG_BLOCK && A.variant == 1) {

@@ -70,7 +70,7 @@ __device__ __forceinline__ void lower_bounds(const float* a, int n, int top, con
 // count_within for two arrays at once: na = #{p : |fl(a[p] - c)| < e} in the
 // ascending a[0..n), nb = the same for (b, d).  The predicates are those of
 // count_within and monotone in p, so the counts are identical.
-__device__ __forceinline__ void count_within_pair(const float* __restrict__ a, const float* __restrict__ b,
+__device__ __forceinline__ void count_within_pair(const float* a, const float* b,
                                                   int n, int top, float c, float d, float e, int& na,
                                                   int& nb) {
     int q[4];
@@ -84,7 +84,7 @@ __device__ __forceinline__ void count_within_pair(const float* __restrict__ a, c
 // The non-strict counts of KSG algorithm 2 for two arrays at once, by the same
 // searches: na = #{p : |fl(a[p] - c)| <= ea}, nb = #{p : |fl(b[p] - d)| <= eb}
 // (the predicates of count_le).
-__device__ __forceinline__ void count_le_pair(const float* __restrict__ a, const float* __restrict__ b, int n,
+__device__ __forceinline__ void count_le_pair(const float* a, const float* b, int n,
                                               int top, float c, float ea, float d, float eb, int& na,
                                               int& nb) {
     int q[4];

@@ -27,6 +27,7 @@
 #include <numeric>
 #include <vector>
 
+#include "device_common.cuh"
 #include "gemm_f32.h"
 #include "hash_common.cuh"
 #include "ndf_hash_tc.h"
@@ -45,10 +46,11 @@ constexpr double kFourierInit = 0.1;
 // (one thread per row, measured: 15 us per 8192 rows; this: 6.5 us for all 16,384).
 constexpr int kEmbedRows = 32;
 __global__ void __launch_bounds__(256)
-    hash_embed_kernel(const float* __restrict__ pos0, const float* __restrict__ pos1, int64_t B, int64_t rows,
-                      const float* __restrict__ enc0, const float* __restrict__ enc1, EmbedArgs E,
-                      float* __restrict__ x0) {
+    hash_embed_kernel(const float* pos0, const float* pos1, int64_t B, int64_t rows,
+                      const float* enc0, const float* enc1, EmbedArgs E,
+                      float* x0) {
     extern __shared__ float xs[];  // [32][ld], ld odd: conflict-free by row
+    pdl_launch();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ld = E.din | 1;
     const int64_t r0 = (int64_t)blockIdx.x * kEmbedRows, r = r0 + lane;
     if (r < rows) {
@@ -82,9 +84,11 @@ __global__ void __launch_bounds__(256)
 
 // hash-table gradient: scatter dL/d(embedding) of the hash features, gx[row][ld] from its
 // column 0 on (rows as in hash_embed_kernel), one thread per row and level
-__global__ void hash_embed_backward_kernel(const float* __restrict__ pos0, const float* __restrict__ pos1,
-                                           int64_t B, int64_t rows, const float* __restrict__ gx, int ld,
-                                           EmbedArgs E, float* __restrict__ genc0, float* __restrict__ genc1) {
+__global__ void hash_embed_backward_kernel(const float* pos0, const float* pos1,
+                                           int64_t B, int64_t rows, const float* gx, int ld,
+                                           EmbedArgs E, float* genc0, float* genc1) {
+    pdl_launch();
+    pdl_wait();
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int l = blockIdx.y;
     if (r >= rows) return;
@@ -103,9 +107,11 @@ __global__ void hash_embed_backward_kernel(const float* __restrict__ pos0, const
 
 // z from the two latents (d features each, zr broadcast when zr_stride == 0):
 // product (the paper's merge), sum, |difference|, or concatenation [zr; zq]
-__global__ void merge_kernel(const float* __restrict__ zr, int64_t zr_stride,
-                             const float* __restrict__ zq, int d, int64_t B, int mode,
-                             float* __restrict__ z) {
+__global__ void merge_kernel(const float* zr, int64_t zr_stride,
+                             const float* zq, int d, int64_t B, int mode,
+                             float* z) {
+    pdl_launch();
+    pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)d * B) return;
     const int64_t b = i / d, o = i - b * d;
@@ -118,9 +124,11 @@ __global__ void merge_kernel(const float* __restrict__ zr, int64_t zr_stride,
     }
 }
 
-__global__ void merge_backward_kernel(const float* __restrict__ g, const float* __restrict__ zr,
-                                      const float* __restrict__ zq, int d, int64_t B, int mode,
-                                      float* __restrict__ gr, float* __restrict__ gq) {
+__global__ void merge_backward_kernel(const float* g, const float* zr,
+                                      const float* zq, int d, int64_t B, int mode,
+                                      float* gr, float* gq) {
+    pdl_launch();
+    pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)d * B) return;
     const int64_t b = i / d, o = i - b * d;
@@ -154,13 +162,15 @@ inline int64_t out_chunk(int64_t B) {
     return (c + kOutRows - 1) / kOutRows * kOutRows;
 }
 __global__ void __launch_bounds__(256)
-    hash_out_kernel(const float* __restrict__ in, const float* __restrict__ w, const float* __restrict__ bias,
-                    int cin, int64_t B, int64_t chunk, int measure, const float* __restrict__ target,
-                    float* __restrict__ y, const float* __restrict__ pre, int act, float* __restrict__ dX, float* __restrict__ part,
-                    double* __restrict__ loss) {
+    hash_out_kernel(const float* in, const float* w, const float* bias,
+                    int cin, int64_t B, int64_t chunk, int measure, const float* target,
+                    float* y, const float* pre, int act, float* dX, float* part,
+                    double* loss) {
     __shared__ float gs[kOutRows];
     __shared__ float red[256];
     __shared__ double ls[8];
+    pdl_launch();
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t begin = (int64_t)blockIdx.x * chunk, end = min(begin + chunk, B);
     const int cw = cin > 128 ? 256 : cin > 64 ? 128 : 64, subs = 256 / cw;
@@ -240,9 +250,11 @@ __device__ __forceinline__ void adam_one(float& p, float g, float& m, float& v, 
 // array streamed once (evict-first); the gradient may be the caller's buffer at any alignment
 // (gvec: 16-byte aligned).
 __global__ void __launch_bounds__(256)
-    hash_adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                     float* __restrict__ v, int64_t n, bool gvec, float lr, float b1, float b2, float eps,
+    hash_adam_kernel(float* p, const float* g, float* m,
+                     float* v, int64_t n, bool gvec, float lr, float b1, float b2, float eps,
                      float c1, float c2) {
+    pdl_launch();
+    pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, j = i << 2;
     if (j + 3 < n) {
         float4 P = __ldcs(reinterpret_cast<const float4*>(p) + i), M = __ldcs(reinterpret_cast<const float4*>(m) + i);
@@ -422,6 +434,7 @@ static cudaError_t encode_rows(ndf_hash_model* m, int e, int batch, const float*
     ndf_ctx* ctx = m->ctx;
     const float* enc0 = m->params + L.enc_size * e;
     float* x0 = m->x0 + row0 * L.din;
+    // an ordinary launch: the table reads (__ldg) must not start beside whatever wrote the tables
     hash_embed_kernel<<<blocks_for(rows, kEmbedRows), 256, sizeof(float) * kEmbedRows * (size_t)(L.din | 1),
                         ctx->stream>>>(pos0, pos1, B, rows, enc0, enc0 + L.enc_size * (batch - 1), embed_args(L), x0);
     ctx->launches++;
@@ -466,9 +479,9 @@ static cudaError_t decode_z(ndf_hash_model* m, int64_t B, const float* target, f
         // weights and bias are adjacent in the parameters: one segment
         g.seg[g.count++] = {part, grad + L.dw[k], cin + 1, (int)blocks, 1};
     }
-    hash_out_kernel<<<blocks, 256, 0, ctx->stream>>>(in, m->params + L.dw[k], m->params + L.db[k], cin, B, chunk,
-                                                     m->measure, target, y, k > 0 ? m->pre_d[k - 1] : nullptr, L.act, m->ga, part,
-                                                     m->loss);
+    launch_after(hash_out_kernel, dim3(blocks), dim3(256), 0, ctx->stream, in, m->params + L.dw[k],
+                 m->params + L.db[k], cin, B, chunk, m->measure, target, y, k > 0 ? m->pre_d[k - 1] : nullptr,
+                 L.act, m->ga, part, m->loss);
     ctx->launches++;
     return cudaGetLastError();
 }
@@ -486,7 +499,8 @@ static cudaError_t hash_forward_backward(ndf_hash_model* m, const float* pr, con
     cudaError_t e = encode_rows(m, 0, batch, pr, pq, B, 2 * B, 0);
     if (e != cudaSuccess) return e;
     const float *zr = latent(m, 0), *zq = latent(m, B);
-    merge_kernel<<<blocks_for((int64_t)L.dlat * B), 256, 0, s>>>(zr, L.dlat, zq, L.dlat, B, L.merge, m->z);
+    launch_after(merge_kernel, dim3(blocks_for((int64_t)L.dlat * B)), dim3(256), 0, s, zr, L.dlat, zq, L.dlat,
+                 B, L.merge, m->z);
     ctx->launches++;
     if ((e = decode_z(m, B, target, y, grad)) != cudaSuccess || !target) return e;
     // ---- backward: decoder (ping-pong ga / gb), merge, then the encoder chain
@@ -498,8 +512,8 @@ static cudaError_t hash_forward_backward(ndf_hash_model* m, const float* pr, con
         if (e != cudaSuccess) return e;
         std::swap(cur, other);
     }
-    merge_backward_kernel<<<blocks_for((int64_t)L.dlat * B), 256, 0, s>>>(cur, zr, zq, L.dlat, B, L.merge, m->gl,
-                                                                          m->gl + B * L.dlat);
+    launch_after(merge_backward_kernel, dim3(blocks_for((int64_t)L.dlat * B)), dim3(256), 0, s, cur, zr, zq,
+                 L.dlat, B, L.merge, m->gl, m->gl + B * L.dlat);
     ctx->launches++;
     const float* gs = m->gl;
     cur = m->ga;
@@ -514,9 +528,9 @@ static cudaError_t hash_forward_backward(ndf_hash_model* m, const float* pr, con
         std::swap(cur, other);
     }
     const bool grid_only = L.le == 0;
-    hash_embed_backward_kernel<<<dim3(blocks_for(2 * B), (unsigned)L.levels), 256, 0, s>>>(
-        pr, pq, B, 2 * B, grid_only ? gs + col0 : gs, grid_only ? L.din : L.din - col0, embed_args(L), grad,
-        grad + L.enc_size * (L.n_enc - 1));
+    launch_after(hash_embed_backward_kernel, dim3(blocks_for(2 * B), (unsigned)L.levels), dim3(256), 0, s, pr,
+                 pq, B, 2 * B, grid_only ? gs + col0 : gs, grid_only ? L.din : L.din - col0, embed_args(L),
+                 grad, grad + L.enc_size * (L.n_enc - 1));
     ctx->launches++;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return grad_sums_flush(s, g, &ctx->launches);
@@ -682,8 +696,8 @@ static cudaError_t hash_fp32_decode(ndf_hash_model* m, int64_t ref_idx, float* d
         ctx->launches++;
         e = encode_rows(m, L.n_enc - 1, 1, pq, pq, n, n, chunk);
         if (e != cudaSuccess) break;
-        merge_kernel<<<blocks_for((int64_t)L.dlat * n), 256, 0, ctx->stream>>>(
-            zr, 0, latent(m, chunk), L.dlat, n, L.merge, m->z);
+        launch_after(merge_kernel, dim3(blocks_for((int64_t)L.dlat * n)), dim3(256), 0, ctx->stream, zr, 0,
+                     latent(m, chunk), L.dlat, n, L.merge, m->z);
         ctx->launches++;
         e = decode_z(m, n, nullptr, dev_out + v0, nullptr);
     }
@@ -821,8 +835,9 @@ static cudaError_t hash_adam(ndf_hash_model* m, const float* grad, float lr) {
     ++m->t;
     ++m->ver;
     const float c1 = 1.0f - powf(0.9f, (float)m->t), c2 = 1.0f - powf(0.999f, (float)m->t);
-    hash_adam_kernel<<<blocks_for((m->Ly.total + 3) / 4), 256, 0, m->ctx->stream>>>(
-        m->params, grad, m->m, m->v, m->Ly.total, ((uintptr_t)grad & 15) == 0, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
+    launch_after(hash_adam_kernel, dim3(blocks_for((m->Ly.total + 3) / 4)), dim3(256), 0, m->ctx->stream,
+                 m->params, grad, m->m, m->v, m->Ly.total, ((uintptr_t)grad & 15) == 0, lr, 0.9f, 0.999f,
+                 1e-8f, c1, c2);
     m->ctx->launches++;
     return cudaGetLastError();
 }
