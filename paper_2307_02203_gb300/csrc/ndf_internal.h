@@ -155,14 +155,16 @@ cudaError_t launch_sort_columns(ndf_ctx* ctx, const Field& f, int64_t v_begin, i
                                 cudaStream_t stream, const float* src = nullptr,
                                 int* d_nonfinite = nullptr);
 
+constexpr int kSampleRows = 4096;  // buckets of grid rows that the sampler orders positions by
 // Scratch of the continuous sampler: position, column and statistics blocks for
 // up to `cap` pairs, reused across calls.
 struct SampleScratch {
     float *ca = nullptr, *cb = nullptr, *cb_sorted = nullptr;
     double *ma = nullptr, *sa = nullptr, *mb = nullptr, *sb = nullptr;
+    int* order = nullptr;  // counts of kSampleRows grid rows, then the positions in their order
     int64_t cap = 0, M = 0;
     void release() {
-        void* ps[] = {ca, cb, cb_sorted, ma, sa, mb, sb};
+        void* ps[] = {ca, cb, cb_sorted, ma, sa, mb, sb, order};
         for (void* q : ps)
             if (q) cudaFree(q);
         *this = SampleScratch();
@@ -177,6 +179,7 @@ struct SampleScratch {
         if (e == cudaSuccess) e = cudaMalloc(&sa, sizeof(double) * (size_t)n);
         if (e == cudaSuccess) e = cudaMalloc(&mb, sizeof(double) * (size_t)n);
         if (e == cudaSuccess) e = cudaMalloc(&sb, sizeof(double) * (size_t)n);
+        if (e == cudaSuccess) e = cudaMalloc(&order, sizeof(int) * ((size_t)n + kSampleRows));
         if (e != cudaSuccess) {
             release();
             return e;

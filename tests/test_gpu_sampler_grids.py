@@ -38,3 +38,26 @@ def test_targets_on_ragged_grids(ndf_mod, ctx, X, Y, Z):
         mi = oracle.ksg_pair(oracle.interp_column(f, pr[i]), oracle.interp_column(f, pq[i]), k)[0]
         assert abs(t[i] - mi) <= 1e-6 * abs(mi) + 1e-9, (i, t[i], mi)
     ndf_mod.ndf_free_ensemble(ctx, fid)
+
+
+@pytest.mark.parametrize("X,Y,Z,n", [(200, 164, 1, 8191), (200, 164, 1, 8192), (217, 151, 1, 9000), (8, 70, 70, 9001),
+                                     (32768, 1, 1, 8200), (40, 30, 2, 9000)])
+def test_positions_in_row_order(ndf_mod, ctx, X, Y, Z, n):
+    """From 8192 positions and 32,768 vertices on they are interpolated in the order of their grid rows
+    (here also more rows than its buckets, a single one, and sizes just outside): every target stays
+    with its pair."""
+    M, k = 20, 2
+    f = np.random.default_rng(n).normal(size=(M, Z, Y, X)).astype(np.float32)
+    g = np.random.default_rng(n + 1).normal(size=(M, Z, Y, X)).astype(np.float32)
+    fa = ndf_mod.ndf_load_ensemble(ctx, f, M, Z, Y, X)
+    fb = ndf_mod.ndf_load_ensemble(ctx, g, M, Z, Y, X)
+    pr, pq, t = np.empty((n, 3), np.float32), np.empty((n, 3), np.float32), np.empty(n, np.float32)
+    ndf_mod.ndf_sample_triples(ctx, fa, fb, ndf_mod.NDF_MEASURE_MI_KSG, k, n, 78, pr, pq, t)
+    want = positions(n, 78)
+    np.testing.assert_array_equal(pr, want[0])
+    np.testing.assert_array_equal(pq, want[1])
+    for i in [*range(0, n, 17), n - 1]:
+        mi = oracle.ksg_pair(oracle.interp_column(f, pr[i]), oracle.interp_column(g, pq[i]), k)[0]
+        assert abs(t[i] - mi) <= 1e-6 * abs(mi) + 1e-9, (i, t[i], mi)
+    ndf_mod.ndf_free_ensemble(ctx, fa)
+    ndf_mod.ndf_free_ensemble(ctx, fb)
