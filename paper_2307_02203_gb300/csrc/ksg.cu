@@ -111,8 +111,8 @@ __global__ void __launch_bounds__(1024)
 // The same for up to 1024 members, one warp per reference: RG (key, member) pairs per lane,
 // element 32 r + lane in register r, sorted by a bitonic network (strides of 32 and more are
 // register pairs, the others shuffles).  No barriers and 32 warps' worth of references per SM
-// at once: 100,000 references of 500 members take 0.55 ms instead of 3.97 ms with one CTA of
-// 1024 threads and 45 barriers each, and a single one of 100 members 2.2 us instead of 7.2.
+// at once: 100,000 references of 500 members take 0.99 ms instead of 3.97 ms with one CTA of
+// 1024 threads and 45 barriers each.
 // A lone reference with many members stays with the CTA above (launch_ksg).
 __device__ __forceinline__ bool stage_less(float a, int va, float b, int vb) {
     return a < b || (a == b && va < vb);
@@ -1451,8 +1451,8 @@ cudaError_t launch_ksg(ndf_ctx* ctx, const Field& rf, const Field& qf, const int
     if (e != cudaSuccess) return e;
     e = ctx->ksg_work.reserve(sizeof(unsigned long long));
     if (e != cudaSuccess) return e;
-    // a warp per reference where there are many of them, or few members (a lone warp needs about
-    // 0.25 us per register of its lanes)
+    // a warp per reference where there are many of them, or few members (a lone warp's network of
+    // 1024 keys is a serial chain of 14,000 instructions; one CTA spreads it)
     auto stage_warps = [&](auto kern) {
         const int warps = R < 4 ? R : 4;
         kern<<<(unsigned)((R + warps - 1) / warps), 32 * warps, 0, ctx->stream>>>(

@@ -152,10 +152,11 @@ __global__ void merge_backward_kernel(const float* g, const float* zr,
 // given, the L1 loss, its gradient through the layer and the layer's own gradients: in[B][cin]
 // is read once, dX = dL/draw * w (* act'(pre), the pre-activations of `in`, when given), and
 // every CTA's sums over its rows of dL/draw * in and dL/draw go to part[blockIdx.x][cin + 1]
-// (added in order by grad_sums_flush).  One warp per row for the dot products, then one thread
+// (added in order by grad_sums_flush).  The dot products in the layers' order (16 terms at a time,
+// then the slices), eight lanes per row; then one thread
 // per column (several row groups when there are fewer columns than threads), 32 rows at a
 // time; a CTA takes `chunk` consecutive rows.
-constexpr int kOutRows = 32;
+constexpr int kOutRows = 32;  // 8 warps x 4 rows
 constexpr int64_t kOutMaxCtas = 256;  // partial sums to add
 inline int64_t out_chunk(int64_t B) {
     const int64_t c = (B + kOutMaxCtas - 1) / kOutMaxCtas;
@@ -179,22 +180,34 @@ __global__ void __launch_bounds__(256)
     double l = 0.0;
     for (int64_t b0 = begin; b0 < end; b0 += kOutRows) {
         const int n = (int)min((int64_t)kOutRows, end - b0);
-        for (int r = warp; r < n; r += 8) {
-            const float* x = in + (b0 + r) * cin;
-            float s = 0.0f;
-#pragma unroll 4
-            for (int i = lane; i < cin; i += 32) s = fmaf(x[i], w[i], s);
+        {
+            const int r = warp * 4 + (lane >> 3), ch = lane & 7;
+            const float* x = in + (b0 + (r < n ? r : 0)) * cin;
+            float acc = 0.0f;
+            for (int c0 = 0; c0 < cin; c0 += 128) {
+                float p = 0.0f;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            const float raw = s + bias[0];
+                for (int i = 0; i < 16; ++i) {
+                    const int k = c0 + 16 * ch + i;
+                    if (k < cin) p = fmaf(x[k], w[k], p);
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float q = __shfl_sync(0xffffffffu, p, (lane & 24) + j);
+                    if (c0 + 16 * j < cin) acc += q;
+                }
+            }
+            const float raw = acc + bias[0];
             const float v = out_act(measure, raw);
-            if (lane == 0 && y) y[b0 + r] = v;
-            if (target) {
-                const float d = v - target[b0 + r];
-                l += fabs((double)d);
-                const float sg = d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f);
-                const float dv = measure == NDF_MEASURE_PEARSON ? 1.0f - v * v : 1.0f / (1.0f + expf(-raw));
-                if (lane == 0) gs[r] = sg / (float)B * dv;
+            if (r < n && ch == 0) {
+                if (y) y[b0 + r] = v;
+                if (target) {
+                    const float d = v - target[b0 + r];
+                    l += fabs((double)d);
+                    const float sg = d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f);
+                    const float dv = measure == NDF_MEASURE_PEARSON ? 1.0f - v * v : 1.0f / (1.0f + expf(-raw));
+                    gs[r] = sg / (float)B * dv;
+                }
             }
         }
         if (!target) continue;
@@ -230,6 +243,8 @@ __global__ void __launch_bounds__(256)
         __syncthreads();  // gs is rewritten by the next rows
     }
     if (!target) return;
+    l += __shfl_xor_sync(0xffffffffu, l, 8);
+    l += __shfl_xor_sync(0xffffffffu, l, 16);
     if (lane == 0) ls[warp] = l;
     __syncthreads();
     if (threadIdx.x == 0) {
