@@ -381,8 +381,8 @@ cudaError_t dense_forward(cudaStream_t s, const DenseLayer& L, const float* X, f
                         pre, post, act, aligned16(X, L.cin), wv, yv);
 }
 
-int64_t dense_grad_floats(int64_t cin, int64_t cout) {
-    return 2 * (kGradSplits * cout * (cin + 1) + 8);
+int64_t dense_grad_floats(int64_t cin, int64_t cout, int batch) {
+    return batch * kGradSplits * cout * (cin + 1) + 16;
 }
 
 cudaError_t grad_sums_flush(cudaStream_t s, GradSums& g, uint64_t* launches) {

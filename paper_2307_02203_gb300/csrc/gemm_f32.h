@@ -47,8 +47,8 @@ struct GradSums {
         return r;
     }
 };
-// workspace one layer needs (any rows, batch of up to two weight sets)
-int64_t dense_grad_floats(int64_t cin, int64_t cout);
+// workspace one layer needs (any rows)
+int64_t dense_grad_floats(int64_t cin, int64_t cout, int batch);
 // adds every listed partial to its destination and empties the list (counts one launch)
 cudaError_t grad_sums_flush(cudaStream_t s, GradSums& g, uint64_t* launches);
 

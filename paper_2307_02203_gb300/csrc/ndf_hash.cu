@@ -400,10 +400,17 @@ static cudaError_t hash_workspace(ndf_hash_model* m, int64_t B) {
     // partial sums of the weight gradients: all layers where that stays within 128 MB (then one
     // kernel adds them all at the end of a step), at least the largest one
     const int64_t out_part = kOutMaxCtas * (std::max<int64_t>(L.ddec, c) + 1);
-    const int64_t one = std::max(std::max(dense_grad_floats(wmax, c), dense_grad_floats(L.ddec, c)), out_part + 4);
-    const int64_t all = (L.le + L.ld) * dense_grad_floats(wmax, c) + out_part + 4;
+    const int64_t enc = L.le > 0 ? dense_grad_floats(std::max<int64_t>(L.din, c), c, L.n_enc) : 0;
+    const int64_t dec = dense_grad_floats(std::max<int64_t>(L.ddec, c), c, 1);
+    const int64_t one = std::max(std::max(enc, dec), out_part + 4);
+    const int64_t all = L.le * enc + L.ld * dec + out_part + 4;
     m->sums.cap = std::max(one, std::min<int64_t>(all, int64_t(32) << 20));
     e = cudaMalloc(&m->sums.work, sizeof(float) * (size_t)m->sums.cap);
+    if (e == cudaErrorMemoryAllocation && m->sums.cap > one) {  // the layers' sums one by one then
+        cudaGetLastError();
+        m->sums.cap = one;
+        e = cudaMalloc(&m->sums.work, sizeof(float) * (size_t)one);
+    }
     if (e != cudaSuccess) {
         m->sums = GradSums();
         return e;
