@@ -214,11 +214,11 @@ ndf_status ndf_mi_ksg2(ndf_ctx* ctx, int ref_field, int query_field, int64_t ref
  *                   blocks outward in x and, inside a block, outward in y, both
  *                   stopped by its current k-th distance (exact pruning).
  *                   Algorithm 1 only: ndf_mi_ksg2 runs NDF_KSG_PRUNED instead;
- *   NDF_KSG_LANES   (default) the same two-level search scheduled per lane: each lane walks
+ *   NDF_KSG_LANES   (default) the same two-level search scheduled per lane, in blocks of
+ *                   32, 64 or 128 x-ranks by M: each lane walks
  *                   its own member's blocks and takes the pair's next member when
  *                   its member is finished; block switches and refills run in a
- *                   shared service step (ndf_ksg_set_schedule).
- *                   Algorithm 1 only, like NDF_KSG_BLOCK;
+ *                   shared service step (ndf_ksg_set_schedule);
  *   NDF_KSG_BRUTE   every member against every member of each pair.
  * count_evals != 0 makes the kernels count distance evaluations (read with
  * ndf_ksg_take_eval_count); it costs one atomic per warp per launch. */

@@ -15,7 +15,6 @@
 // slots so that one slot's epilogue overlaps the other slot's MMAs:
 //   warps 0-7 (slot 0) and 8-15 (slot 1): thread i of a slot's two halves owns row i of the
 //     tile (TMEM lane i) and 64 of its columns.  The halves encode the vertex once per tile
-//     tile (TMEM lane i) and 64 of its columns.  The halves encode the vertex once per tile
 //     (two levels each; 64 FP32 features in shared memory); then for each reference, after
 //     each layer, they load their columns of the FP32 accumulator with tcgen05.ld, add the
 //     bias, round, apply ReLU and write the next layer's operand (after layer 3 the columns stay as BF16
@@ -32,8 +31,9 @@
 // so what counts is what stands between a commit and the next hand-over (with x, dot product and
 // output there too it was 2,900 cycles after layer 3, and 3,800 per layer with one warp per 128
 // columns and operands in shared memory).  16 references on 1.76M vertices: 4.29 ms before,
-// 2.90 ms now (3.66 with the biases in shared memory).  (The biases as a ninth K step of three BF16 terms each: 2.83 ms, but the sums before
-// the rounding to BF16 are then added in another order.)
+// 2.90 ms now (3.66 with the biases in shared memory; with the biases as a ninth K step of
+// three BF16 terms each 2.83 ms, but the sums before the rounding to BF16 are then added in another
+// order.)
 // The references' features f(p_r) (FP32) sit in shared memory, the biases in constant memory.
 #include <cuda_bf16.h>
 
