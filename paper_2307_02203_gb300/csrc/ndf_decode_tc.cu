@@ -433,7 +433,6 @@ void const_slot_release(int device, int slot) {
 cudaError_t launch_infer_tc(ndf_model* m, const int64_t* d_refs, int R, float* out) {
     ndf_ctx* ctx = m->ctx;
     // from 100,000 values on (40 us) the constant copy after a parameter update (2 us) is repaid by
-    // its first call
     // its first call; a captured call reads the parameters themselves (its copy would not run now)
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(ctx->stream, &capture);
@@ -449,8 +448,13 @@ cudaError_t launch_infer_tc(ndf_model* m, const int64_t* d_refs, int R, float* o
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(static_cast<char*>(base) + (size_t)m->cslot * sizeof(c_net[0]), m->mlp_vec(),
                                 sizeof(c_net[0]), cudaMemcpyDeviceToDevice, ctx->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(m->cslot_ready, ctx->stream);
         if (e != cudaSuccess) return e;
         m->cslot_stale = false;
+    } else if (constant) {
+        // the copy may have run on another stream, which this call need not follow
+        e = cudaStreamWaitEvent(ctx->stream, m->cslot_ready, 0);
+        if (e != cudaSuccess) return e;
     }
     TcInferArgs a;
     a.G.grid = m->grid_bf;

@@ -322,6 +322,11 @@ ndf_status model_alloc(ndf_ctx* ctx, const int res[kLevels], int measure, int64_
         return cuda_fail(ctx, e, "model allocation");
     }
     m->cslot = const_slot_acquire(ctx->device);
+    if (m->cslot >= 0 && cudaEventCreateWithFlags(&m->cslot_ready, cudaEventDisableTiming) != cudaSuccess) {
+        (void)cudaGetLastError();
+        const_slot_release(m->ctx->device, m->cslot);
+        m->cslot = -1;  // the decoder then reads the parameters themselves
+    }
     *out = m;
     return NDF_OK;
 }
@@ -332,6 +337,7 @@ void model_free(ndf_model* m) {
     for (void* q : ps)
         if (q) cudaFree(q);
     m->work.release();
+    if (m->cslot_ready) cudaEventDestroy(m->cslot_ready);
     const_slot_release(m->ctx->device, m->cslot);
     delete m;
 }

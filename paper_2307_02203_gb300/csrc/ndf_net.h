@@ -65,6 +65,7 @@ struct ndf_model {
     float* mlp_vec() const { return reinterpret_cast<float*>(wbf + 3 * 128 * 128); }  // b1, b2, b3, w4
     int cslot = -1;             // the decoder's constant-memory slot of mlp_vec (-1: none)
     bool cslot_stale = true;    // mlp_vec has changed since it was copied there
+    cudaEvent_t cslot_ready = nullptr;  // after that copy: a decode may run on another stream
     int64_t t = 0;             // Adam steps taken
     ndf::NetWork work;
     // training record

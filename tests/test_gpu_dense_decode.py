@@ -103,3 +103,28 @@ def test_constant_memory_slots(ndf_mod, ctx):
     np.testing.assert_array_equal(volumes(models[-2]), first[19])
     for m in models:
         ndf_mod.ndf_model_free(m)
+
+
+def test_constant_memory_on_two_streams(ndf_mod, ctx):
+    """The first decode after an update fills the model's constant memory on its own stream; the next
+    one, on another stream that does not wait for the first, reads the same values."""
+    X, Y, Z = 50, 50, 20
+    m = ndf_mod.ndf_model_create(ctx, RES_SMALL, 0, 2, X, Y, Z)
+    ndf_mod.ndf_model_set_params(m, make_params(5))
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    out = torch.zeros((2, 2, X * Y * Z), device="cuda")
+    torch.cuda.synchronize()
+    try:
+        with torch.cuda.stream(streams[0]):
+            torch.cuda._sleep(20_000_000)
+        for s, o in zip(streams, out):
+            ndf_mod.ndf_set_stream(ctx, s.cuda_stream)
+            ndf_mod.ndf_infer_batch(m, [3, 777], o)
+        torch.cuda.synchronize()
+    finally:
+        ndf_mod.ndf_set_stream(ctx, None)
+    np.testing.assert_array_equal(out[1].cpu().numpy(), out[0].cpu().numpy())
+    one = np.empty(X * Y * Z, np.float32)
+    ndf_mod.ndf_infer(m, 3, one)
+    np.testing.assert_array_equal(out[1, 0].cpu().numpy(), one)
+    ndf_mod.ndf_model_free(m)
