@@ -32,6 +32,14 @@ inline cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
+// Lifts a kernel's dynamic shared memory limit to the most a CTA can have, whatever the launch at
+// hand needs: the limit belongs to the function and the device, so a smaller one set for one
+// thread's launch would refuse another thread's larger launch that is about to follow.
+constexpr size_t kMaxDynamicSmem = 227 * 1024;
+template <class Kern>
+inline cudaError_t allow_dynamic_smem(Kern kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamicSmem);
+}
 
 // Bit flags of the device status word (ctx->flag, word 1).
 enum : unsigned { kDevTimeout = 1u, kDevBadInput = 2u };

@@ -1340,7 +1340,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
 template <class Kern>
 static cudaError_t launch_persistent(ndf_ctx* ctx, Kern kern, const KsgArgs& A, int threads,
                                     size_t smem, int64_t items) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(kern);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
@@ -1362,7 +1362,7 @@ static cudaError_t launch_ksg_k(ndf_ctx* ctx, KsgArgs A, bool prune) {
         const size_t per_group = (size_t)LaneSmem(M, lw).total;
         const size_t shared_x = A.R == 1 ? sizeof(float) * (size_t)M : 0;
         const int64_t pairs = A.paired ? (A.v_end - A.v_begin) : (int64_t)A.R * (A.v_end - A.v_begin);
-        int gpc = (int)((227 * 1024 - shared_x) / per_group);
+        int gpc = (int)((kMaxDynamicSmem - shared_x) / per_group);
         if (gpc > kLaneMaxGroups) gpc = kLaneMaxGroups;
         // fewer pairs than the chip's groups: one CTA per SM, with as few groups as that needs
         const int64_t need = (pairs + ctx->sm_count - 1) / ctx->sm_count;
@@ -1371,7 +1371,7 @@ static cudaError_t launch_ksg_k(ndf_ctx* ctx, KsgArgs A, bool prune) {
             const size_t smem = (size_t)gpc * per_group + shared_x;
             const int threads = 32 * kGroupWarps * gpc;
             auto kern = ksg_lane_kernel<K1>;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = allow_dynamic_smem(kern);
             if (e != cudaSuccess) return e;
             int64_t grid = (int64_t)ctx->sm_count;
             if (grid * gpc > pairs) grid = (pairs + gpc - 1) / gpc;
@@ -1384,13 +1384,13 @@ static cudaError_t launch_ksg_k(ndf_ctx* ctx, KsgArgs A, bool prune) {
     if (prune && ctx->ksg_algorithm == NDF_KSG_BLOCK && A.variant == 1) {
         // two-warp groups per pair; as many groups per CTA as fit in shared memory
         const size_t per_group = block_group_bytes(M);
-        int gpc = (int)((227 * 1024) / per_group);
+        int gpc = (int)(kMaxDynamicSmem / per_group);
         if (gpc > kMaxGroupsPerCta) gpc = kMaxGroupsPerCta;
         if (gpc >= 1) {
             const size_t smem = (size_t)gpc * per_group;
             const int threads = 32 * kGroupWarps * gpc;
             auto kern = ksg_block_kernel<K1>;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = allow_dynamic_smem(kern);
             if (e != cudaSuccess) return e;
             const int64_t pairs = A.paired ? (A.v_end - A.v_begin) : (int64_t)A.R * (A.v_end - A.v_begin);
             int64_t grid = (int64_t)ctx->sm_count;
@@ -1403,13 +1403,13 @@ static cudaError_t launch_ksg_k(ndf_ctx* ctx, KsgArgs A, bool prune) {
     if (prune) {
         // one warp group per pair; as many groups per CTA as fit in shared memory
         const size_t per_group = (size_t)kGroupSmemPerM * M + kGroupSmemFixed;
-        int gpc = (int)((227 * 1024) / per_group);
+        int gpc = (int)(kMaxDynamicSmem / per_group);
         if (gpc > kMaxGroupsPerCta) gpc = kMaxGroupsPerCta;
         if (gpc < 1) gpc = 1;
         const size_t smem = (size_t)gpc * per_group;
         const int threads = 32 * kGroupWarps * gpc;
         auto kern = ksg_pruned_kernel<K1>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_dynamic_smem(kern);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);

@@ -483,13 +483,11 @@ static ndf_status gemm_chunk(ndf_ctx* ctx, const Field& rf, const Field& qf, boo
     int grid = ctx->sm_count;
     if (grid > ntiles) grid = (int)ntiles;
     if (bf16) {
-        e = cudaFuncSetAttribute(pearson_gemm_kernel<true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_dynamic_smem(pearson_gemm_kernel<true>);
         if (e == cudaSuccess)
             pearson_gemm_kernel<true><<<grid, kGemmThreads, smem, ctx->stream>>>(mA, mA2, mB, mB2, g);
     } else {
-        e = cudaFuncSetAttribute(pearson_gemm_kernel<false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_dynamic_smem(pearson_gemm_kernel<false>);
         if (e == cudaSuccess)
             pearson_gemm_kernel<false><<<grid, kGemmThreads, smem, ctx->stream>>>(mA, mA2, mB, mB2, g);
     }
