@@ -219,7 +219,8 @@ struct KsgArgs {
     const float* xs_all;  // [R][M] sorted reference values
     const int* perm_all;  // [R][M] member id of each sorted position
     const double* psi;    // psi(n), n <= M + 1
-    const long long* psi_fix;  // the same in fixed point (kPsiFixBits)
+    const long long* psi_fix;  // the same in fixed point, with M's bits (psi_fix_bits)
+    double psi_scale;     // 2^-bits
     float* out;           // out[r * out_stride + (v - v_begin)]
     int64_t out_stride;
     int variant;          // KSG algorithm 1 or 2
@@ -1327,7 +1328,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
                 sum += ctl->part[w];
                 gave_up = gave_up || ctl->part[w] == LLONG_MIN;
             }
-            const double tot = (double)sum * (1.0 / (double)(1ll << kPsiFixBits));
+            const double tot = (double)sum * A.psi_scale;
             double mi = psi_k - (A.variant == 2 ? 1.0 / A.k : 0.0) + psi_M - tot / (double)M;
             if (gave_up) mi = __longlong_as_double(0x7ff8000000000000ll);
             A.out[A.paired ? (v - A.v_begin) : (int64_t)r * A.out_stride + (v - A.v_begin)] = (float)mi;
@@ -1483,7 +1484,9 @@ cudaError_t launch_ksg(ndf_ctx* ctx, const Field& rf, const Field& qf, const int
     A.xs_all = ctx->stage_x.as<float>();
     A.perm_all = ctx->stage_perm.as<int>();
     A.psi = ctx->psi.as<double>();
-    A.psi_fix = reinterpret_cast<const long long*>(A.psi + ctx->psi_n);
+    const int group = psi_fix_group(M);
+    A.psi_fix = reinterpret_cast<const long long*>(A.psi + ctx->psi_n) + psi_fix_offset(group);
+    A.psi_scale = 1.0 / (double)(1ll << psi_fix_bits(group));
     A.out = out;
     A.out_stride = out_stride;
     A.dbg_mi = dbg_mi;

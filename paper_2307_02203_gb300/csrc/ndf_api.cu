@@ -207,18 +207,19 @@ double digamma_int_host(int64_t n) {
 ndf_status ensure_psi_table(ndf_ctx* ctx, int64_t n_max) {
     if (ctx->psi_n > n_max) return NDF_OK;
     int64_t n = n_max + 1;
-    // n doubles, then the same values in fixed point
+    // n doubles, then the fixed-point copies of every group up to n_max members
+    const int groups = psi_fix_group((int)n_max);
     std::vector<double> h((size_t)n, 0.0);
-    std::vector<int64_t> fix((size_t)n, 0);
-    for (int64_t i = 1; i < n; ++i) {
-        h[(size_t)i] = digamma_int_host(i);
-        fix[(size_t)i] = (int64_t)llrint(ldexp(h[(size_t)i], kPsiFixBits));
-    }
-    const size_t bytes = sizeof(double) * (size_t)n;
-    cudaError_t e = ctx->psi.reserve(2 * bytes);
+    std::vector<int64_t> fix((size_t)psi_fix_offset(groups + 1), 0);
+    for (int64_t i = 1; i < n; ++i) h[(size_t)i] = digamma_int_host(i);
+    for (int g = 1; g <= groups; ++g)
+        for (int64_t i = 1; i <= (int64_t)1 << g && i < n; ++i)
+            fix[(size_t)(psi_fix_offset(g) + i)] = (int64_t)llrint(ldexp(h[(size_t)i], psi_fix_bits(g)));
+    const size_t bytes = sizeof(double) * (size_t)n, fix_bytes = sizeof(int64_t) * fix.size();
+    cudaError_t e = ctx->psi.reserve(bytes + fix_bytes);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->psi.ptr, h.data(), bytes, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ctx->psi.as<double>() + n, fix.data(), bytes, cudaMemcpyHostToDevice, ctx->stream);
+        e = cudaMemcpyAsync(ctx->psi.as<double>() + n, fix.data(), fix_bytes, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "digamma table upload");
     ctx->psi_n = n;
