@@ -381,8 +381,8 @@ cudaError_t dense_forward(cudaStream_t s, const DenseLayer& L, const float* X, f
                         pre, post, act, aligned16(X, L.cin), wv, yv);
 }
 
-int64_t dense_grad_floats(int64_t cin, int64_t cout, int batch) {
-    return batch * kGradSplits * cout * (cin + 1) + 16;
+int64_t dense_grad_floats(int64_t cin, int64_t cout, int64_t rows, int batch, int64_t max_splits) {
+    return batch * dense_grad_splits(rows, max_splits) * cout * (cin + 1) + 16;
 }
 
 cudaError_t grad_sums_flush(cudaStream_t s, GradSums& g, uint64_t* launches) {
@@ -408,9 +408,7 @@ cudaError_t dense_backward(cudaStream_t s, const DenseLayer& L, const float* X, 
                            uint64_t* launches) {
     if (L.rows <= 0 || L.cout <= 0 || L.cin <= 0) return cudaSuccess;
     BackwardArgs a;
-    // chunks of at least 128 rows (eight slices, the length of a 128-wide data-gradient tile)
-    int64_t splits = (L.rows + 127) / 128;
-    if (splits > kGradSplits) splits = kGradSplits;
+    const int64_t splits = dense_grad_splits(L.rows, g.max_splits);
     a.chunk = ((L.rows + splits - 1) / splits + kBK - 1) / kBK * kBK;
     a.splits = (int)((L.rows + a.chunk - 1) / a.chunk);
     const int64_t wn = (int64_t)L.cin * L.cout, sb = (int64_t)a.splits * L.batch;

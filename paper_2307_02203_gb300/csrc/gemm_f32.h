@@ -38,6 +38,8 @@ struct GradSeg {
 struct GradSums {
     float* work = nullptr;
     int64_t cap = 0, used = 0;
+    int64_t rows = 0;  // the batch that it was sized for
+    int64_t max_splits = kGradSplits;
     GradSeg seg[kGradSegs];
     int count = 0;
     float* take(int64_t floats) {  // nullptr: flush first
@@ -47,8 +49,14 @@ struct GradSums {
         return r;
     }
 };
-// workspace one layer needs (any rows)
-int64_t dense_grad_floats(int64_t cin, int64_t cout, int batch);
+// chunks of a layer's rows: of at least 128 rows (eight slices, the length of a 128-wide
+// data-gradient tile), at most max_splits of them
+inline int64_t dense_grad_splits(int64_t rows, int64_t max_splits) {
+    const int64_t s = (rows + 127) / 128;
+    return s < 1 ? 1 : s > max_splits ? max_splits : s;
+}
+// workspace one layer needs for up to `rows` rows of each of its `batch` weight sets
+int64_t dense_grad_floats(int64_t cin, int64_t cout, int64_t rows, int batch, int64_t max_splits);
 // adds every listed partial to its destination and empties the list (counts one launch)
 cudaError_t grad_sums_flush(cudaStream_t s, GradSums& g, uint64_t* launches);
 

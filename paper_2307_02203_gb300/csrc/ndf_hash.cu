@@ -357,9 +357,7 @@ namespace ndf {
 static cudaError_t hash_workspace(ndf_hash_model* m, int64_t B) {
     if (B <= m->cap) return cudaSuccess;
     if (m->ws) cudaFree(m->ws);
-    if (m->sums.work) cudaFree(m->sums.work);
     m->ws = nullptr;
-    m->sums = GradSums();
     m->cap = 0;
     const HashLayout& L = m->Ly;
     const int64_t c = L.c, wmax = std::max<int64_t>(std::max<int64_t>(L.din, c), L.ddec);
@@ -397,25 +395,40 @@ static cudaError_t hash_workspace(ndf_hash_model* m, int64_t B) {
     if (e != cudaSuccess) return e;
     m->ws = o;
     carve();
-    // partial sums of the weight gradients: all layers where that stays within 128 MB (then one
-    // kernel adds them all at the end of a step), at least the largest one
-    const int64_t out_part = kOutMaxCtas * (std::max<int64_t>(L.ddec, c) + 1);
-    const int64_t enc = L.le > 0 ? dense_grad_floats(std::max<int64_t>(L.din, c), c, L.n_enc) : 0;
-    const int64_t dec = dense_grad_floats(std::max<int64_t>(L.ddec, c), c, 1);
-    const int64_t one = std::max(std::max(enc, dec), out_part + 4);
-    const int64_t all = L.le * enc + L.ld * dec + out_part + 4;
-    m->sums.cap = std::max(one, std::min<int64_t>(all, int64_t(32) << 20));
-    e = cudaMalloc(&m->sums.work, sizeof(float) * (size_t)m->sums.cap);
-    if (e == cudaErrorMemoryAllocation && m->sums.cap > one) {  // the layers' sums one by one then
-        cudaGetLastError();
-        m->sums.cap = one;
-        e = cudaMalloc(&m->sums.work, sizeof(float) * (size_t)one);
+    m->cap = B;
+    return cudaSuccess;
+}
+
+// The weight gradients' partial sums for batches of up to B pairs (a step's alone: a forward call
+// or a decode takes none): all layers where that stays within 128 MB (then one kernel adds them
+// all at the end of a step), at least the largest one; with memory too short for that, fewer and
+// longer chunks of rows.
+static cudaError_t hash_grad_workspace(ndf_hash_model* m, int64_t B) {
+    if (B <= m->sums.rows) return cudaSuccess;
+    if (m->sums.work) cudaFree(m->sums.work);
+    m->sums = GradSums();
+    const HashLayout& L = m->Ly;
+    const int64_t c = L.c, out_blocks = std::min<int64_t>((B + kOutRows - 1) / kOutRows, kOutMaxCtas);
+    const int64_t out_part = out_blocks * (std::max<int64_t>(L.ddec, c) + 1) + 4;
+    cudaError_t e = cudaErrorMemoryAllocation;
+    for (int64_t splits = kGradSplits; splits >= 1 && e == cudaErrorMemoryAllocation; splits /= 2) {
+        const int64_t enc =
+            L.le > 0 ? dense_grad_floats(std::max<int64_t>(L.din, c), c, 2 * B / L.n_enc, L.n_enc, splits) : 0;
+        const int64_t dec = dense_grad_floats(std::max<int64_t>(L.ddec, c), c, B, 1, splits);
+        const int64_t one = std::max(std::max(enc, dec), out_part), all = L.le * enc + L.ld * dec + out_part;
+        m->sums.max_splits = splits;
+        for (int64_t cap : {std::max(one, std::min<int64_t>(all, int64_t(32) << 20)), one}) {
+            m->sums.cap = cap;
+            e = cudaMalloc(&m->sums.work, sizeof(float) * (size_t)cap);
+            if (e != cudaErrorMemoryAllocation) break;
+            cudaGetLastError();
+        }
     }
     if (e != cudaSuccess) {
         m->sums = GradSums();
         return e;
     }
-    m->cap = B;
+    m->sums.rows = B;
     return cudaSuccess;
 }
 
@@ -882,6 +895,7 @@ ndf_status ndf_hash_model_step(ndf_hash_model* m, const float* pr, const float* 
     ndf_ctx* ctx = m->ctx;
     cudaSetDevice(ctx->device);
     cudaError_t e = hash_workspace(m, B);
+    if (e == cudaSuccess) e = hash_grad_workspace(m, B);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "hash workspace");
     const size_t pb = sizeof(float) * 3 * (size_t)B;
     e = cudaMemcpyAsync(m->pos, pr, pb, cudaMemcpyDefault, ctx->stream);
@@ -1004,6 +1018,7 @@ ndf_status ndf_hash_train(ndf_ctx* ctx, int ref_field, int query_field, int meas
     if (e == cudaSuccess) e = cudaMalloc(&pq, sizeof(float) * 3 * (size_t)T);
     if (e == cudaSuccess) e = cudaMalloc(&tgt, sizeof(float) * (size_t)T);
     if (e == cudaSuccess) e = hash_workspace(m, B);
+    if (e == cudaSuccess) e = hash_grad_workspace(m, B);
     SampleScratch sc;
     auto cleanup = [&]() {
         if (pref) cudaFree(pref);
