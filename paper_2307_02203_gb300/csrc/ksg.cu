@@ -39,6 +39,8 @@
 #include <limits.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "device_common.cuh"
 #include "ksg_common.cuh"
 #include "ndf_internal.h"
@@ -738,51 +740,34 @@ __device__ __forceinline__ int block_lower_bound(const float2* blk, float y) {
     return pos;
 }
 
-// KSG algorithm 2 over the block layout: the largest fl(|x_j - xi|) and fl(|y_j - yi|)
+// KSG algorithm 2 over the lane search's blocks: the largest fl(|x_j - xi|) and fl(|y_j - yi|)
 // over the members j whose max-norm distance to (xi, yi) is <= e (the member itself adds
 // zeros).  Blocks from the member's own block b0 outward in x while the block's nearest
-// x-rank is within e (fl(x_j - xi) is monotone in x_j); inside a block, outward in y
-// from the lower bound of yi while |dy| <= e (the +inf separators stop both scans).
-__device__ __forceinline__ void block_extents(const float2* blk, const float2* bx, int M, int nb, int lw,
-                                              int b0, float xi, float yi, float e, float& ex, float& ey) {
+// x-rank is within e (fl(x_j - xi) is monotone in x_j); inside a block, outward in y while
+// |dy| <= e (the +inf separators stop both scans), from the member's own position p0 there and
+// from enter(block) = the number of members below yi elsewhere.
+template <class Enter>
+__device__ __forceinline__ void block_extents(const float2* blk, const float2* bx, int nb, int bs, int b0, int p0,
+                                              float xi, float yi, float e, float& ex, float& ey, Enter&& enter) {
     ex = 0.0f;
     ey = 0.0f;
-    auto scan = [&](int bb) {
-        const float2* B = blk + 1 + bb * ((1 << lw) + 1);  // (y, x), ascending y
-        int pos = 0;
-        for (int len = min(1 << lw, M - (bb << lw)); len > 0;) {  // members below yi
-            const int h = len >> 1;
-            if (B[pos + h].x < yi) {
-                pos += h + 1;
-                len -= h + 1;
-            } else {
-                len = h;
-            }
+    auto visit = [&](const float2* c) {  // false: beyond e in y
+        const float dy = fabsf(c->x - yi), dx = fabsf(c->y - xi);
+        if (!(dy <= e)) return false;
+        if (dx <= e) {
+            ex = fmaxf(ex, dx);
+            ey = fmaxf(ey, dy);
         }
-        for (int u = pos;; ++u) {
-            const float2 c = B[u];
-            const float dy = fabsf(c.x - yi);
-            if (!(dy <= e)) break;
-            const float dx = fabsf(c.y - xi);
-            if (dx <= e) {
-                ex = fmaxf(ex, dx);
-                ey = fmaxf(ey, dy);
-            }
-        }
-        for (int u = pos - 1;; --u) {
-            const float2 c = B[u];
-            const float dy = fabsf(yi - c.x);
-            if (!(dy <= e)) break;
-            const float dx = fabsf(c.y - xi);
-            if (dx <= e) {
-                ex = fmaxf(ex, dx);
-                ey = fmaxf(ey, dy);
-            }
-        }
+        return true;
     };
-    scan(b0);
-    for (int bb = b0 + 1; bb < nb && bx[bb].x - xi <= e; ++bb) scan(bb);
-    for (int bb = b0 - 1; bb >= 0 && xi - bx[bb].y <= e; --bb) scan(bb);
+    auto scan = [&](int bb, int pos) {
+        const float2* B = blk + 1 + bb * bs;  // (y, x), ascending y
+        for (int u = pos; visit(B + u); ++u) {}
+        for (int u = pos - 1; visit(B + u); --u) {}
+    };
+    scan(b0, p0);
+    for (int bb = b0 + 1; bb < nb && bx[bb].x - xi <= e; ++bb) scan(bb, enter(bb));
+    for (int bb = b0 - 1; bb >= 0 && xi - bx[bb].y <= e; --bb) scan(bb, enter(bb));
 }
 
 template <int K1>
@@ -1022,23 +1007,21 @@ struct LaneSmem {
     }
 };
 // ranks per block: the scan visits members inside the y-window of whole blocks, so wider blocks
-// cost candidates that fail the x-test, narrower ones more block switches.  Measured (ms a
-// volume, 32 / 64 / 128 ranks): 1.118 / 1.157 / 1.384 for M = 200, k = 4 (88,000 vertices);
-// 0.440 / 0.437 / 0.466 for M = 333, k = 5 (18,361); 1.88 / 1.74 / 1.95 for M = 600, k = 6
-// (40,000); 10.5 / 7.6 / 6.9 for M = 1000, k = 8 (88,000); 6.7 / 4.2 / 3.5 for M = 1800, k = 10
-// (14,400).
-__host__ __device__ inline int lane_block_log2(int M) { return M > 768 ? 7 : M > 256 ? 6 : 5; }
+// cost candidates that fail the x-test, narrower ones more block switches.  Measured (us a volume of
+// 1.2e7 / M vertices, k = 8, 32 / 64 / 128 ranks): 1073 / 1080 / 1375 for M = 200, 973 / 935 / 1264 for
+// M = 256, 1139 / 962 / 1030 for M = 600, 1166 / 981 / 1021 for M = 769, 1296 / 1086 / 1073 for M = 900,
+// 1336 / 1131 / 1018 for M = 1000.
+__host__ __device__ inline int lane_block_log2(int M) { return M > 850 ? 7 : M > 224 ? 6 : 5; }
 // lock steps a warp may take per pair before it gives up (a safety bound far above
 // any real schedule: every member visits at most nb blocks of W + 1 steps)
 __host__ __device__ inline long long lane_step_bound(int nb, int lw) {
     return (long long)lane_slots(nb, lw) * (nb + 2) * ((1 << lw) + 4);
 }
-constexpr int kLaneMaxGroups = 13;  // groups per CTA: what shared memory holds at M = 1000
-constexpr int kLaneMaxRegs = 4;  // ranks per lane of a block (W <= 128; `below` counts in bytes)
-
-template <int K1>
+constexpr int kLaneMaxGroups = 14;  // groups per CTA: the most that leave a thread 72 registers
+// RPL: ranks per lane of the widest block (W <= 32 RPL)
+template <int K1, int RPL>
 __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
-    ksg_lane_kernel(KsgArgs A, unsigned long long* work, int lw, int switch_min, int every) {
+    ksg_lane_kernel(KsgArgs A, unsigned long long* work, int lw, bool x_shared, int switch_min, int every) {
     constexpr int KK = K1 - 1;
     constexpr int GT = 32 * kGroupWarps;
     constexpr unsigned FULL = 0xffffffffu;
@@ -1061,11 +1044,9 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
     const int64_t N = A.N, nv = A.v_end - A.v_begin;
     const unsigned long long items =
         A.paired ? (unsigned long long)nv : (unsigned long long)A.R * (unsigned long long)nv;
-    const double psi_k = A.psi[A.k], psi_M = A.psi[M];
     const int step_bound = (int)min(lane_step_bound(nb, lw), (long long)INT_MAX);
     const int top = pow2_floor(M);
     unsigned long long evals_total = 0;
-    const bool x_shared = A.R == 1;
     float* xsh = reinterpret_cast<float*>(smem + (blockDim.x / GT) * L.total);
     if (x_shared) {
         for (int i = threadIdx.x; i < M; i += blockDim.x) xsh[i] = A.xs_all[i];
@@ -1149,18 +1130,20 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
                     const int u = __shfl_up_sync(FULL, inc, o);
                     inc += lane >= o ? u : 0;
                 }
-                if (w < nw) bb[w] = (unsigned char)(carry + inc - c);
+                // 256 ranks below a word count as 255: its word is empty then, and a scan that enters
+                // there starts one rank lower and sees the same members
+                if (w < nw) bb[w] = (unsigned char)(RPL > 4 ? min(carry + inc - c, 255) : carry + inc - c);
                 carry += __shfl_sync(FULL, inc, 31);
             }
-            int rk[kLaneMaxRegs];
+            int rk[RPL];
 #pragma unroll
-            for (int j = 0; j < kLaneMaxRegs; ++j) {
+            for (int j = 0; j < RPL; ++j) {
                 const int s = (b << lw) + j * 32 + lane;
                 rk[j] = j * 32 < W && s < M ? rank_s[s] : -1;
             }
             __syncwarp();  // the counts are written, the ranks read (their places are reused)
 #pragma unroll
-            for (int j = 0; j < kLaneMaxRegs; ++j) {
+            for (int j = 0; j < RPL; ++j) {
                 if (rk[j] < 0) continue;
                 const int s = (b << lw) + j * 32 + lane;
                 const int pos = bb[rk[j] >> 5] + __popc(tb[rk[j] >> 5] & ((1u << (rk[j] & 31)) - 1u));
@@ -1276,7 +1259,13 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
             int cx, cy;
             if (A.variant == 2) {  // non-strict counts within the k-NN set's marginal extents
                 float ex, ey;
-                block_extents(blk, bx, M, nb, lw, b, me.y, me.x, e, ex, ey);
+                const float yq[1] = {me.x};
+                int rank[1];  // the query column's members below
+                lower_bounds<1>(ys, M, top, yq, rank);
+                const int w = min(rank[0], M - 1) >> 5;
+                const unsigned under = (1u << (rank[0] & 31)) - 1u;
+                block_extents(blk, bx, nb, bs, b, pos - (b << lw), me.y, me.x, e, ex, ey,
+                              [&](int bb) { return below[bb * nw + w] + __popc(tab[bb * nw + w] & under); });
                 count_le_pair(xsg, ys, M, top, me.y, ex, me.x, ey, cx, cy);
                 --cx;  // the member itself excluded
                 --cy;
@@ -1329,7 +1318,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
                 gave_up = gave_up || ctl->part[w] == LLONG_MIN;
             }
             const double tot = (double)sum * A.psi_scale;
-            double mi = psi_k - (A.variant == 2 ? 1.0 / A.k : 0.0) + psi_M - tot / (double)M;
+            double mi = A.psi[A.k] - (A.variant == 2 ? 1.0 / A.k : 0.0) + A.psi[M] - tot / (double)M;
             if (gave_up) mi = __longlong_as_double(0x7ff8000000000000ll);
             A.out[A.paired ? (v - A.v_begin) : (int64_t)r * A.out_stride + (v - A.v_begin)] = (float)mi;
             if (dbg && A.dbg_mi) *A.dbg_mi = mi;
@@ -1354,30 +1343,54 @@ static cudaError_t launch_persistent(ndf_ctx* ctx, Kern kern, const KsgArgs& A, 
     return cudaGetLastError();
 }
 
+// How the lane search runs a call: 2^lw ranks per block, gpc groups per CTA, the reference in shared
+// memory or not (algorithm 1 alone reads it there).  The usual form is lane_block_log2's width with
+// the shared reference, and 13 groups from 257 members on (14 against 13 groups, us for 1.2e7 / M
+// vertices, k = 4: 1126 / 1159 for M = 60, 645 / 645 for M = 256, 733 / 703 for M = 600).  Another form may
+// place another group per SM: the 14th, the reference left in global memory, blocks of 256 ranks, which halve
+// the bitmaps.  It is taken where that saves a round of pairs: above 1700 members always (k = 8, 128
+// against 256 ranks: 1509 / 1393 for M = 1800, 2268 / 1829 for M = 3000; M = 4096, without the reference,
+// 4372 / 3292; where no group is gained 128 is the better one, M = 3500, k = 4: 2107 / 2146, algorithm 2: 3858
+// / 4000), below where it saves at least a fifth of the rounds (2100 vertices, M = 500, k = 8: 136 in two
+// rounds, 100 in one; 1600 vertices, M = 1200: 347 and 249).
+struct LanePlan {
+    int lw, gpc;
+    bool x_shared;
+};
+static LanePlan lane_plan(int M, int64_t pairs, int sms, bool x_shared) {
+    const int64_t need = (pairs + sms - 1) / sms;  // groups per SM that take all pairs at once
+    auto groups = [&](int lw, bool xs, int most) {
+        const int64_t g = (int64_t)((kMaxDynamicSmem - (xs ? sizeof(float) * (size_t)M : 0)) / LaneSmem(M, lw).total);
+        return (int)std::min(std::min<int64_t>(g, most), need);
+    };
+    auto rounds = [&](int gpc) { return gpc > 0 ? (need + gpc - 1) / gpc : need + 1; };
+    LanePlan best = {lane_block_log2(M), 0, x_shared};
+    best.gpc = groups(best.lw, best.x_shared, M > 256 ? kLaneMaxGroups - 1 : kLaneMaxGroups);
+    const LanePlan other[4] = {{best.lw, 0, x_shared}, {best.lw, 0, false}, {8, 0, x_shared}, {8, 0, false}};
+    for (LanePlan o : other) {
+        o.gpc = groups(o.lw, o.x_shared, kLaneMaxGroups);
+        if ((M > 1700 ? 4 : 5) * rounds(o.gpc) < 4 * rounds(best.gpc)) best = o;
+    }
+    return best;
+}
+
 template <int K1>
 static cudaError_t launch_ksg_k(ndf_ctx* ctx, KsgArgs A, bool prune) {
     const int M = A.M;
     if (prune && ctx->ksg_algorithm == NDF_KSG_LANES && (A.variant == 1 || A.variant == 2)) {
-        // two-warp groups per pair; as many groups per CTA as fit in shared memory
-        const int lw = lane_block_log2(M);
-        const size_t per_group = (size_t)LaneSmem(M, lw).total;
-        const size_t shared_x = A.R == 1 ? sizeof(float) * (size_t)M : 0;
+        // two-warp groups per pair
         const int64_t pairs = A.paired ? (A.v_end - A.v_begin) : (int64_t)A.R * (A.v_end - A.v_begin);
-        int gpc = (int)((kMaxDynamicSmem - shared_x) / per_group);
-        if (gpc > kLaneMaxGroups) gpc = kLaneMaxGroups;
-        // fewer pairs than the chip's groups: one CTA per SM, with as few groups as that needs
-        const int64_t need = (pairs + ctx->sm_count - 1) / ctx->sm_count;
-        if (gpc > need) gpc = (int)need;
-        if (gpc >= 1) {
-            const size_t smem = (size_t)gpc * per_group + shared_x;
-            const int threads = 32 * kGroupWarps * gpc;
-            auto kern = ksg_lane_kernel<K1>;
+        const LanePlan p = lane_plan(M, pairs, ctx->sm_count, A.R == 1 && A.variant == 1);
+        if (p.gpc >= 1) {
+            const size_t smem = (size_t)p.gpc * LaneSmem(M, p.lw).total + (p.x_shared ? sizeof(float) * (size_t)M : 0);
+            const int threads = 32 * kGroupWarps * p.gpc;
+            auto kern = p.lw > 7 ? ksg_lane_kernel<K1, 8> : ksg_lane_kernel<K1, 4>;
             cudaError_t e = allow_dynamic_smem(kern);
             if (e != cudaSuccess) return e;
             int64_t grid = (int64_t)ctx->sm_count;
-            if (grid * gpc > pairs) grid = (pairs + gpc - 1) / gpc;
+            if (grid * p.gpc > pairs) grid = (pairs + p.gpc - 1) / p.gpc;
             e = launch_after(kern, dim3((unsigned)grid), dim3((unsigned)threads), smem, ctx->stream, A,
-                             ctx->ksg_work.as<unsigned long long>(), lw, ctx->ksg_switch_min, ctx->ksg_every);
+                             ctx->ksg_work.as<unsigned long long>(), p.lw, p.x_shared, ctx->ksg_switch_min, ctx->ksg_every);
             ctx->launches++;
             return e;
         }
