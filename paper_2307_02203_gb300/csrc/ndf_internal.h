@@ -180,8 +180,8 @@ struct SampleScratch {
             if (q) cudaFree(q);
         *this = SampleScratch();
     }
-    cudaError_t reserve(int64_t M_, int64_t n) {
-        if (n <= cap && M_ == M) return cudaSuccess;
+    cudaError_t reserve(int64_t M_, int64_t n, bool ordered) {
+        if (n <= cap && M_ == M && (order || !ordered)) return cudaSuccess;
         release();
         cudaError_t e = cudaMalloc(&ca, sizeof(float) * (size_t)M_ * (size_t)n);
         if (e == cudaSuccess) e = cudaMalloc(&cb, sizeof(float) * (size_t)M_ * (size_t)n);
@@ -190,7 +190,7 @@ struct SampleScratch {
         if (e == cudaSuccess) e = cudaMalloc(&sa, sizeof(double) * (size_t)n);
         if (e == cudaSuccess) e = cudaMalloc(&mb, sizeof(double) * (size_t)n);
         if (e == cudaSuccess) e = cudaMalloc(&sb, sizeof(double) * (size_t)n);
-        if (e == cudaSuccess) e = cudaMalloc(&order, sizeof(int) * ((size_t)n + kSampleRows));
+        if (e == cudaSuccess && ordered) e = cudaMalloc(&order, sizeof(int) * ((size_t)n + kSampleRows));
         if (e != cudaSuccess) {
             release();
             return e;

@@ -152,8 +152,8 @@ __global__ void sample_order_kernel(const float* __restrict__ pos, int64_t n, in
 }
 
 // VEC (N and the base 16-byte aligned): the two x-neighbours of a row come from one aligned
-// 16-byte load (three positions in four) or that and a 4-byte one, not two 4-byte ones: every
-// lane's row is another sector, so the kernel is bound by the requests, not by the bytes.
+// 16-byte load (three positions in four) or that and a 4-byte one, not two 4-byte ones: fewer requests,
+// a longer chain.
 template <bool VEC>
 __global__ void interp_columns_kernel(const float* __restrict__ field, int64_t M, int64_t X,
                                       int64_t Y, int64_t Z, const float* __restrict__ pos, const int* __restrict__ order,
@@ -226,11 +226,21 @@ __global__ void make_batch_pos_kernel(const float* __restrict__ pref, const floa
     target[i] = tgt[j];
 }
 
-// Positions are ordered from this many on, on grids whose level of one member does not stay in an
-// SM's L1 anyway.  Measured (us, unordered / ordered): 100,000 KSG triples of 500 members on 440,000
-// vertices 7,638 / 7,059; 200,000 Pearson triples of 1000 members on 50,000 vertices 10,816 / 9,031,
-// of 100 members on 4,500 vertices 1,436 / 1,639; 20,000 of 500 members on 440,000 1,177 / 1,107.
-constexpr int64_t kSampleOrderMin = 8192, kSampleOrderVertices = 32768;
+// Positions are ordered where the columns they are interpolated to have this many values: the
+// interpolation gains with positions times members, the ordering costs 25 us and grows with the
+// positions.  Measured (us, unordered / ordered, Pearson triples): 8192 of 1000 members on 110,000 vertices
+// 1240 / 1202, 65,536 of them 3987 / 3089; 16,384 of 300 on 40,000 676 / 632; 4000 of 500 on 440,000 789 /
+// 819; 65,536 of 60 on 440,000 622 / 649.  Twice as many on small grids, of which one member's level
+// stays in an SM's L1: 32,768 on 4500 vertices of 200 members 602 / 618, of 300 755 / 743.
+constexpr int64_t kSampleSmallGrid = 32768;
+static bool sample_ordered(int64_t n, int64_t M, int64_t N) { return n * M >= (N < kSampleSmallGrid ? 8000000 : 4000000); }
+// The x-neighbours in pairs only on those small grids, for 1000 positions and more that are not ordered
+// (us, two loads / paired: 4000 of 60 members on 4500 vertices 240 / 233, 1000 of 300 446 / 434; but 300
+// of 1000 members on 110,000 vertices 957 / 978, a single one of 200 121 / 125, and 65,536 ordered
+// ones of 1000 3090 / 3298).
+static bool sample_paired(int64_t n, const Field& f) {
+    return n >= 1000 && f.N < kSampleSmallGrid && (f.N & 3) == 0 && ((uintptr_t)f.data & 15) == 0;
+}
 
 // n triples (p_ref, p_q, R(p_ref, p_q)) at uniform random positions in [-1,1]^3
 // (Sec. 4.3), written to device arrays pref[n][3], pq[n][3], target[n].  Pairs
@@ -240,7 +250,7 @@ cudaError_t sample_triples_dev(ndf_ctx* ctx, const Field& rf, const Field& qf, i
                                SampleScratch& sc) {
     const int64_t M = rf.M;
     const int64_t chunk = std::min<int64_t>(n, 65536);
-    cudaError_t e = sc.reserve(M, chunk);
+    cudaError_t e = sc.reserve(M, chunk, sample_ordered(chunk, M, std::max(rf.N, qf.N)));
     if (e != cudaSuccess) return e;
     const uint64_t key = host_mix(seed ^ 0x434f4e54504f5353ULL);
     int* d_flag = ctx->flag.as<int>();
@@ -251,9 +261,10 @@ cudaError_t sample_triples_dev(ndf_ctx* ctx, const Field& rf, const Field& qf, i
         const dim3 grid((unsigned)((nc + 127) / 128), (unsigned)std::min<int64_t>(M, 64));
         auto interp = [&](const Field& f, const float* pos, float* out) {
             const int* order = nullptr;
-            if (nc >= kSampleOrderMin && f.N >= kSampleOrderVertices) {
+            if (sample_ordered(nc, M, f.N)) {
                 int *count = sc.order, *sorted = sc.order + kSampleRows;
-                cudaMemsetAsync(count, 0, sizeof(int) * kSampleRows, ctx->stream);
+                e = cudaMemsetAsync(count, 0, sizeof(int) * kSampleRows, ctx->stream);
+                if (e != cudaSuccess) return;
                 const unsigned blocks = (unsigned)((nc + 255) / 256);
                 sample_count_kernel<<<blocks, 256, 0, ctx->stream>>>(pos, nc, f.Y, f.Z, count);
                 sample_scan_kernel<<<1, kSampleRows / 4, 0, ctx->stream>>>(count);
@@ -261,13 +272,12 @@ cudaError_t sample_triples_dev(ndf_ctx* ctx, const Field& rf, const Field& qf, i
                 ctx->launches += 3;
                 order = sorted;
             }
-            if ((f.N & 3) == 0 && ((uintptr_t)f.data & 15) == 0)
-                interp_columns_kernel<true><<<grid, 128, 0, ctx->stream>>>(f.data, M, f.X, f.Y, f.Z, pos, order, nc, out);
-            else
-                interp_columns_kernel<false><<<grid, 128, 0, ctx->stream>>>(f.data, M, f.X, f.Y, f.Z, pos, order, nc, out);
+            auto kern = !order && sample_paired(nc, f) ? interp_columns_kernel<true> : interp_columns_kernel<false>;
+            kern<<<grid, 128, 0, ctx->stream>>>(f.data, M, f.X, f.Y, f.Z, pos, order, nc, out);
         };
         interp(rf, pref + 3 * c0, sc.ca);
-        interp(qf, pq + 3 * c0, sc.cb);
+        if (e == cudaSuccess) interp(qf, pq + 3 * c0, sc.cb);
+        if (e != cudaSuccess) break;
         ctx->launches += 3;
         Field fa, fb;
         fa.live = fb.live = true;
