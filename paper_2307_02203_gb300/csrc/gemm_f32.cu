@@ -336,10 +336,9 @@ __global__ void __launch_bounds__(kThreads, 2) dense_backward_kernel(DenseLayer 
 
 struct GradSegs {
     GradSeg s[kGradSegs];
-    int count;
 };
 
-// dst[i] (+)= the sum of part[0 .. splits)[i]: a CTA of 32 columns and 8 row lanes (a warp reads 32
+// dst[i] += the sum of part[0 .. splits)[i]: a CTA of 32 columns and 8 row lanes (a warp reads 32
 // consecutive columns of one partial); lane y sums the partials y, y + 8, .. in order, then the
 // lanes' sums are added in order.  blockIdx.y: segment
 __global__ void __launch_bounds__(256) grad_sums_kernel(GradSegs g) {
@@ -361,7 +360,7 @@ __global__ void __launch_bounds__(256) grad_sums_kernel(GradSegs g) {
             float t = 0.0f;
 #pragma unroll
             for (int y = 0; y < 8; ++y) t += red[y][tx];
-            s.dst[i] = s.add ? s.dst[i] + t : t;
+            s.dst[i] += t;
         }
         __syncthreads();
     }
@@ -393,7 +392,6 @@ cudaError_t grad_sums_flush(cudaStream_t s, GradSums& g, uint64_t* launches) {
         k.s[i] = g.seg[i];
         if (g.seg[i].n > nmax) nmax = g.seg[i].n;
     }
-    k.count = g.count;
     int64_t bx = (nmax + 31) / 32;
     if (bx > 4096) bx = 4096;
     ++*launches;
@@ -420,8 +418,8 @@ cudaError_t dense_backward(cudaStream_t s, const DenseLayer& L, const float* X, 
     a.bpart = g.take(sb * L.cout);
     if (!a.wpart || !a.bpart) return cudaErrorInvalidValue;  // the workspace holds one layer
     for (int z = 0; z < L.batch; ++z) {
-        g.seg[g.count++] = {a.wpart + z * a.splits * wn, dW + z * L.wstride, wn, a.splits, 1};
-        g.seg[g.count++] = {a.bpart + (int64_t)z * a.splits * L.cout, db + z * L.wstride, L.cout, a.splits, 1};
+        g.seg[g.count++] = {a.wpart + z * a.splits * wn, dW + z * L.wstride, wn, a.splits};
+        g.seg[g.count++] = {a.bpart + (int64_t)z * a.splits * L.cout, db + z * L.wstride, L.cout, a.splits};
     }
     a.X = X;
     a.dY = dY;

@@ -30,10 +30,9 @@ constexpr int kGradSegs = 40;
 constexpr int64_t kGradSplits = 64;   // most chunks of one layer
 struct GradSeg {
     const float* part;  // [splits][n]
-    float* dst;         // dst[i] (+)= sum over the splits
+    float* dst;         // dst[i] += sum over the splits
     int64_t n;
     int splits;
-    int add;
 };
 struct GradSums {
     float* work = nullptr;

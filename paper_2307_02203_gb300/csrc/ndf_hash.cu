@@ -288,11 +288,6 @@ __global__ void __launch_bounds__(256)
     for (int64_t k = j; k < n; ++k) adam_one(p[k], g[k], m[k], v[k], lr, b1, b2, eps, c1, c2);
 }
 
-__global__ void fill_kernel(float* __restrict__ p, int64_t n, float v) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
-}
-
 __global__ void vertex_positions_kernel(int64_t v0, int64_t n, int64_t X, int64_t Y, int64_t Z,
                                         float* __restrict__ pos) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -512,7 +507,7 @@ static cudaError_t decode_z(ndf_hash_model* m, int64_t B, const float* target, f
         part = g.take((int64_t)blocks * (cin + 1));
         if (!part) return cudaErrorInvalidValue;  // the list is empty here and holds one layer
         // weights and bias are adjacent in the parameters: one segment
-        g.seg[g.count++] = {part, grad + L.dw[k], cin + 1, (int)blocks, 1};
+        g.seg[g.count++] = {part, grad + L.dw[k], cin + 1, (int)blocks};
     }
     launch_after(hash_out_kernel, dim3(blocks), dim3(256), 0, ctx->stream, in, m->params + L.dw[k],
                  m->params + L.db[k], cin, B, chunk, m->measure, target, y, k > 0 ? m->pre_d[k - 1] : nullptr,

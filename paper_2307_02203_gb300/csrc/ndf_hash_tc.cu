@@ -13,20 +13,16 @@
 //                 merge -> decoder runs per reference
 //
 // CTA roles (one CTA per SM, persistent over 128-vertex tiles):
-//   warps 0-7 / 8-15: two tile slots.  Row i of a slot's tile (TMEM lane i) belongs
-//     to two warps: warp q + 4 h of the slot (q = i / 32) owns its columns
-//     64 h .. 64 h + 63.  Half 0 writes the position and Fourier features of the
-//     row's vertex into the slot's A tile (BF16, 128-byte-swizzled K-major), half 1
-//     the hash-grid features; after each layer each half reads its 64 accumulator
-//     columns with tcgen05.ld, adds the bias, applies the activation (or the
-//     merge) with packed FP32x2 arithmetic and writes them back as the next
-//     layer's A operand.  The output layer's two half dot products meet through
-//     shared memory (an mbarrier per slot).
-//   warp 16: allocates TMEM (2 x 128 columns); one lane issues the MMAs, layer by
-//     layer for both slots, and commits to the slot's mbarrier and, once both
+//   warps 0-15: four tile slots of four warps.  Row i of a slot's tile (TMEM lane i) belongs
+//     to one thread.  It writes the embedding of the row's vertex into the slot's A tile
+//     (BF16, 128-byte-swizzled K-major); after each layer it reads its 128 accumulator
+//     columns with tcgen05.ld, adds the bias, applies the activation (or the merge) with
+//     packed FP32x2 arithmetic and writes them back as the next layer's A operand.
+//   warp 16: allocates TMEM (4 x 128 columns); one lane issues the MMAs, layer by
+//     layer for the four slots in turn, and commits to the slot's mbarrier and, once all
 //     slots used a weight buffer, to that buffer's "empty" mbarrier.
 //   warp 17: one lane streams the layers' weight images (32 KB each, pre-swizzled
-//     in global memory, L2-resident) into a ring of three shared-memory buffers
+//     in global memory, L2-resident) into a ring of two shared-memory buffers
 //     with cp.async.bulk.
 // All waits are bounded (polls and wall time); on timeout every role stops, the
 // copies in flight are waited for, TMEM is freed and the status word is set.

@@ -40,14 +40,14 @@ __device__ __forceinline__ void vertex_pos(int64_t v, int64_t X, int64_t Y, int6
     p[2] = axis_pos(z, Z);
 }
 
-__host__ __device__ static inline uint64_t host_mix(uint64_t z) {
+__host__ __device__ static inline uint64_t mix64(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
     z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
     return z ^ (z >> 31);
 }
 
-__host__ __device__ static inline uint64_t host_rand(uint64_t key, uint64_t i) {
-    return host_mix(key + (i + 1) * 0x9e3779b97f4a7c15ULL);
+__host__ __device__ static inline uint64_t rand64(uint64_t key, uint64_t i) {
+    return mix64(key + (i + 1) * 0x9e3779b97f4a7c15ULL);
 }
 
 // gather the query columns of one group: out[m][q] = field[m][verts[q]]
@@ -104,7 +104,7 @@ __global__ void sample_positions_kernel(uint64_t key, int64_t c0, int64_t n, flo
     if (i >= n) return;
 #pragma unroll
     for (int d = 0; d < 6; ++d) {
-        const float v = (float)(int)(host_rand(key, (uint64_t)((c0 + i) * 6 + d)) >> 40) * 0x1.0p-23f - 1.0f;
+        const float v = (float)(int)(rand64(key, (uint64_t)((c0 + i) * 6 + d)) >> 40) * 0x1.0p-23f - 1.0f;
         if (d < 3) pref[3 * i + d] = v;
         else pq[3 * i + d - 3] = v;
     }
@@ -252,7 +252,7 @@ cudaError_t sample_triples_dev(ndf_ctx* ctx, const Field& rf, const Field& qf, i
     const int64_t chunk = std::min<int64_t>(n, 65536);
     cudaError_t e = sc.reserve(M, chunk, sample_ordered(chunk, M, std::max(rf.N, qf.N)));
     if (e != cudaSuccess) return e;
-    const uint64_t key = host_mix(seed ^ 0x434f4e54504f5353ULL);
+    const uint64_t key = mix64(seed ^ 0x434f4e54504f5353ULL);
     int* d_flag = ctx->flag.as<int>();
     for (int64_t c0 = 0; c0 < n && e == cudaSuccess; c0 += chunk) {
         const int64_t nc = std::min(chunk, n - c0);
@@ -692,13 +692,13 @@ ndf_status ndf_train(ndf_ctx* ctx, int ref_field, int query_field, int measure, 
     }
     std::vector<int64_t> hq((size_t)Qg), hrefs((size_t)Rg);
     std::vector<int32_t> hr((size_t)(cont ? 0 : T)), hqv((size_t)(cont ? 0 : T));
-    const uint64_t key = host_mix(cfg.seed ^ 0x4e44465452414e53ULL);
+    const uint64_t key = mix64(cfg.seed ^ 0x4e44465452414e53ULL);
     int64_t filled = 0, group = 0;
     int* d_flag = ctx->flag.as<int>();
     while (!cont && filled < T && e == cudaSuccess) {
         // queries of this group: Qg distinct-ish uniform vertices, sorted for locality
         for (int64_t q = 0; q < Qg; ++q)
-            hq[(size_t)q] = (int64_t)(host_rand(key, (uint64_t)(group * 2 * Qg + q)) % (uint64_t)N);
+            hq[(size_t)q] = (int64_t)(rand64(key, (uint64_t)(group * 2 * Qg + q)) % (uint64_t)N);
         std::sort(hq.begin(), hq.end());
         e = cudaMemcpyAsync(dq, hq.data(), (size_t)Qg * 8, cudaMemcpyHostToDevice, ctx->stream);
         if (e != cudaSuccess) break;
@@ -716,7 +716,7 @@ ndf_status ndf_train(ndf_ctx* ctx, int ref_field, int query_field, int measure, 
         // reference vertices of this group (as many as the remaining triples need)
         const int64_t rows = std::min<int64_t>(Rg, (T - filled + Qg - 1) / Qg);
         for (int64_t r = 0; r < rows; ++r)
-            hrefs[(size_t)r] = (int64_t)(host_rand(key ^ 0xa5a5a5a5ULL, (uint64_t)(group * Rg + r)) %
+            hrefs[(size_t)r] = (int64_t)(rand64(key ^ 0xa5a5a5a5ULL, (uint64_t)(group * Rg + r)) %
                                          (uint64_t)rf->N);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(drefs, hrefs.data(), (size_t)rows * 8, cudaMemcpyHostToDevice,
@@ -793,10 +793,10 @@ ndf_status ndf_train(ndf_ctx* ctx, int ref_field, int query_field, int measure, 
             if (e != cudaSuccess) break;
         }
         // a new affine bijection j = a*i + c (mod T) every pass
-        uint64_t a = host_rand(key ^ 0x5bd1e995ULL, (uint64_t)pass) % (uint64_t)T;
+        uint64_t a = rand64(key ^ 0x5bd1e995ULL, (uint64_t)pass) % (uint64_t)T;
         if (a == 0) a = 1;
         while (std::gcd(a, (uint64_t)T) != 1) a = (a + 1) % (uint64_t)T == 0 ? 1 : a + 1;
-        const uint64_t c = host_rand(key ^ 0x27d4eb2fULL, (uint64_t)pass) % (uint64_t)T;
+        const uint64_t c = rand64(key ^ 0x27d4eb2fULL, (uint64_t)pass) % (uint64_t)T;
         e = cudaMemsetAsync(m->work.loss, 0, 8, ctx->stream);
         for (int64_t base = 0; base < T && e == cudaSuccess; base += B) {
             const int64_t b = T - base < B ? T - base : B;
