@@ -215,9 +215,10 @@ ndf_status ndf_mi_ksg2(ndf_ctx* ctx, int ref_field, int query_field, int64_t ref
  *                   stopped by its current k-th distance (exact pruning).
  *                   Algorithm 1 only: ndf_mi_ksg2 runs NDF_KSG_PRUNED instead;
  *   NDF_KSG_LANES   (default) the same two-level search scheduled per lane, in blocks of
- *                   32, 64 or 128 x-ranks by M: each lane walks
- *                   its own member's blocks and takes the pair's next member when
- *                   its member is finished; block switches and refills run in a
+ *                   32 to 256 x-ranks by M (and the number of pairs): each lane walks
+ *                   its own member's blocks and takes its warp's next member when
+ *                   its member is finished (a pair's members are split evenly between
+ *                   two warps); block switches and refills run in a
  *                   shared service step (ndf_ksg_set_schedule);
  *   NDF_KSG_BRUTE   every member against every member of each pair.
  * count_evals != 0 makes the kernels count distance evaluations (read with

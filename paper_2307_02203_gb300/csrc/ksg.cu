@@ -1018,6 +1018,121 @@ __host__ __device__ inline long long lane_step_bound(int nb, int lw) {
     return (long long)lane_slots(nb, lw) * (nb + 2) * ((1 << lw) + 4);
 }
 constexpr int kLaneMaxGroups = 14;  // groups per CTA: the most that leave a thread 72 registers
+// The search of one pair by one warp: the joint k-NN distance of each of its members, to eps_s by block
+// position.  gofs: the group's shared memory; returns (evaluations in bytes of points visited, gave up).
+// A function of its own, not inlined: its registers are then allocated apart from those of the
+// kernel's other phases, whose changes moved the scan's code by up to 3 % (88,000 vertices, M = 1000:
+// inlined 7.14 ms with k = 8 and 5.31 with k = 4, as a function 6.80 and 5.13).
+template <int KK>
+__device__ __noinline__ uint2 lane_search(int gofs, int M, int lw, int gw, bool constant, int switch_min, int every) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr unsigned FULL = 0xffffffffu;
+    // five scan steps, the default number, in a row (two: 6.90 ms in the case above, k = 8), but the longer
+    // steps of more neighbours singly (M = 60, 200,000 vertices, k = 10: 1729 us with five)
+    constexpr int kUnroll = KK > 8 ? 1 : 5;
+    const int lane = threadIdx.x & 31;
+    const int W = 1 << lw, nb = (M + W - 1) >> lw, nw = (M + 31) >> 5, bs = W + 1;
+    const LaneSmem L(M, lw);
+    float* eps_s = reinterpret_cast<float*>(smem + gofs + L.eps);
+    const int* rank_s = reinterpret_cast<const int*>(eps_s);
+    const unsigned* tab = reinterpret_cast<const unsigned*>(smem + gofs + L.tab);
+    const unsigned char* below = smem + gofs + L.below;
+    const float2* bx = reinterpret_cast<const float2*>(smem + gofs + L.bx) + 1;
+    const int slots = lane_slots(nb, lw);
+    const int step_bound = (int)min(lane_step_bound(nb, lw), (long long)INT_MAX);
+    const int pt0 = gofs + L.blk + (int)sizeof(float2);  // block 0, position 0
+    bool has = false, inblk = false;
+    int up = pt0 - (int)sizeof(float2), dn = up;  // byte offsets; separators for an idle lane
+    int nr = 0, nl = -1, rank = 0, slot_pos = 0;
+    int next = 0;  // members handed out by this warp (task order, every kGroupWarps-th task)
+    const int wslots = slots / kGroupWarps;
+    float xi = 0.0f, yi = 0.0f;
+    float best[KK];
+#pragma unroll
+    for (int c = 0; c < KK; ++c) best[c] = FLT_MAX;
+    unsigned my_evals = 0;
+    int steps = 0;
+    for (;;) {
+        const unsigned wm = __ballot_sync(FULL, has ? !inblk : next < wslots);
+        const unsigned em = __ballot_sync(FULL, has && inblk);
+        if (em == 0u && wm == 0u) break;
+        if (em == 0u || __popc(wm) >= switch_min) {
+            // service: block switches of the lanes whose window closed, then refills
+            if (has && !inblk) {
+                my_evals += (unsigned)(up - dn);
+                const float t = best[KK - 1];
+                const float x = constant ? yi : xi;
+                const float gr = bx[nr].x - x, gl = x - bx[nl].y;
+                const bool okr = gr < t, okl = gl < t;
+                if (!okr && !okl) {
+                    eps_s[slot_pos] = t;  // member finished
+                    has = false;
+                    my_evals -= (unsigned)sizeof(float2);  // itself
+                    up = dn = pt0 - (int)sizeof(float2);
+                } else {
+                    const bool go_r = okr && (!okl || gr <= gl);
+                    const int cb = go_r ? nr : nl;
+                    nr += go_r ? 1 : 0;
+                    nl -= go_r ? 0 : 1;
+                    const int wd = cb * nw + (rank >> 5);
+                    const int pos = below[wd] + __popc(tab[wd] & ((1u << (rank & 31)) - 1u));
+                    up = pt0 + (cb * bs + pos) * (int)sizeof(float2);
+                    dn = up - (int)sizeof(float2);
+                    inblk = true;
+                }
+                my_evals -= (unsigned)sizeof(float2);
+            }
+            const unsigned dm = __ballot_sync(FULL, !has);
+            if (dm != 0u && next < wslots) {
+                const int q = next + __popc(dm & ((1u << lane) - 1u));
+                next += __popc(dm);
+                // slot q of the warp -> block, position; slots past a block's end are empty
+                const int task = (q >> 5) * kGroupWarps + gw;
+                const int b = ((task >> (lw - 3)) << 2) + ((q >> 3) & 3);
+                const int p = ((task & ((W >> 3) - 1)) << 3) + (q & 7);
+                if (!has && q < wslots && b < nb && (b << lw) + p < M) {
+                    up = pt0 + (b * bs + p) * (int)sizeof(float2);
+                    const float2 me = *reinterpret_cast<const float2*>(smem + up);
+                    yi = me.x;
+                    xi = me.y;
+                    dn = up - (int)sizeof(float2);
+                    up += (int)sizeof(float2);
+                    has = true;
+                    inblk = true;
+                    nr = b + 1;
+                    nl = b - 1;
+                    slot_pos = (b << lw) + p;
+                    rank = rank_s[slot_pos];
+#pragma unroll
+                    for (int c = 0; c < KK; ++c) best[c] = FLT_MAX;
+                }
+            }
+        }
+        steps += every;
+        if (steps > step_bound) break;  // never expected: the pair's MI becomes NaN
+        // `every` scan steps: one candidate above and one below in the lane's current
+        // block (idle lanes, and lanes whose window has closed, re-read candidates at
+        // least the threshold away and leave their lists unchanged)
+        const unsigned long long P = pack_f2(make_float2(yi, xi));
+        bool au = false, ad = false;
+#pragma unroll kUnroll
+        for (int rep = 0; rep < every; ++rep) {
+            const float t = best[KK - 1];
+            const float2 eu = sub_f32x2(P, *reinterpret_cast<const unsigned long long*>(smem + up));
+            const float2 ed = sub_f32x2(P, *reinterpret_cast<const unsigned long long*>(smem + dn));
+            au = fabsf(eu.x) < t;
+            ad = fabsf(ed.x) < t;
+            const float du = fmaxf(fabsf(eu.x), fabsf(eu.y));
+            const float dd = fmaxf(fabsf(ed.x), fabsf(ed.y));
+            insert2<KK>(best, fminf(du, dd), fmaxf(du, dd));
+            up += au ? (int)sizeof(float2) : 0;
+            dn -= ad ? (int)sizeof(float2) : 0;
+        }
+        inblk = au || ad;  // a closed side stays closed: the threshold only shrinks
+    }
+    return make_uint2(my_evals, steps > step_bound ? 1u : 0u);
+}
+
 // RPL: ranks per lane of the widest block (W <= 32 RPL)
 template <int K1, int RPL>
 __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
@@ -1030,7 +1145,6 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
     const int M = A.M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int group = warp / kGroupWarps, gw = warp % kGroupWarps, gt = threadIdx.x % GT;
     const int W = 1 << lw, nb = (M + W - 1) >> lw, nw = (M + 31) >> 5, bs = W + 1;
-    const int slots = lane_slots(nb, lw);
     const LaneSmem L(M, lw);
     unsigned char* gbase = smem + group * L.total;
     LaneCtl* ctl = reinterpret_cast<LaneCtl*>(gbase);
@@ -1044,7 +1158,6 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
     const int64_t N = A.N, nv = A.v_end - A.v_begin;
     const unsigned long long items =
         A.paired ? (unsigned long long)nv : (unsigned long long)A.R * (unsigned long long)nv;
-    const int step_bound = (int)min(lane_step_bound(nb, lw), (long long)INT_MAX);
     const int top = pow2_floor(M);
     unsigned long long evals_total = 0;
     float* xsh = reinterpret_cast<float*>(smem + (blockDim.x / GT) * L.total);
@@ -1156,97 +1269,9 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kLaneMaxGroups, 1)
         group_sync(group);
 
         // ---- joint k-NN distance of every member, lanes refilled from their warp's members
-        const int pt0 = group * L.total + L.blk + (int)sizeof(float2);  // block 0, position 0
-        bool has = false, inblk = false;
-        int up = pt0 - (int)sizeof(float2), dn = up;  // byte offsets; separators for an idle lane
-        int nr = 0, nl = -1, rank = 0, slot_pos = 0;
-        int next = 0;  // members handed out by this warp (task order, every kGroupWarps-th task)
-        const int wslots = slots / kGroupWarps;
-        float xi = 0.0f, yi = 0.0f;
-        float best[KK];
-#pragma unroll
-        for (int c = 0; c < KK; ++c) best[c] = FLT_MAX;
-        unsigned my_evals = 0;
-        int steps = 0;
-        for (;;) {
-            const unsigned wm = __ballot_sync(FULL, has ? !inblk : next < wslots);
-            const unsigned em = __ballot_sync(FULL, has && inblk);
-            if (em == 0u && wm == 0u) break;
-            if (em == 0u || __popc(wm) >= switch_min) {
-                // service: block switches of the lanes whose window closed, then refills
-                if (has && !inblk) {
-                    my_evals += (unsigned)(up - dn);
-                    const float t = best[KK - 1];
-                    const float x = constant ? yi : xi;
-                    const float gr = bx[nr].x - x, gl = x - bx[nl].y;
-                    const bool okr = gr < t, okl = gl < t;
-                    if (!okr && !okl) {
-                        eps_s[slot_pos] = t;  // member finished
-                        has = false;
-                        my_evals -= (unsigned)sizeof(float2);  // itself
-                        up = dn = pt0 - (int)sizeof(float2);
-                    } else {
-                        const bool go_r = okr && (!okl || gr <= gl);
-                        const int cb = go_r ? nr : nl;
-                        nr += go_r ? 1 : 0;
-                        nl -= go_r ? 0 : 1;
-                        const int wd = cb * nw + (rank >> 5);
-                        const int pos = below[wd] + __popc(tab[wd] & ((1u << (rank & 31)) - 1u));
-                        up = pt0 + (cb * bs + pos) * (int)sizeof(float2);
-                        dn = up - (int)sizeof(float2);
-                        inblk = true;
-                    }
-                    my_evals -= (unsigned)sizeof(float2);
-                }
-                const unsigned dm = __ballot_sync(FULL, !has);
-                if (dm != 0u && next < wslots) {
-                    const int q = next + __popc(dm & ((1u << lane) - 1u));
-                    next += __popc(dm);
-                    // slot q of the warp -> block, position; slots past a block's end are empty
-                    const int task = (q >> 5) * kGroupWarps + gw;
-                    const int b = ((task >> (lw - 3)) << 2) + ((q >> 3) & 3);
-                    const int p = ((task & ((W >> 3) - 1)) << 3) + (q & 7);
-                    if (!has && q < wslots && b < nb && (b << lw) + p < M) {
-                        up = pt0 + (b * bs + p) * (int)sizeof(float2);
-                        const float2 me = *reinterpret_cast<const float2*>(smem + up);
-                        yi = me.x;
-                        xi = me.y;
-                        dn = up - (int)sizeof(float2);
-                        up += (int)sizeof(float2);
-                        has = true;
-                        inblk = true;
-                        nr = b + 1;
-                        nl = b - 1;
-                        slot_pos = (b << lw) + p;
-                        rank = rank_s[slot_pos];
-#pragma unroll
-                        for (int c = 0; c < KK; ++c) best[c] = FLT_MAX;
-                    }
-                }
-            }
-            steps += every;
-            if (steps > step_bound) break;  // never expected: the pair's MI becomes NaN
-            // `every` scan steps: one candidate above and one below in the lane's current
-            // block (idle lanes, and lanes whose window has closed, re-read candidates at
-            // least the threshold away and leave their lists unchanged)
-            const unsigned long long P = pack_f2(make_float2(yi, xi));
-            bool au = false, ad = false;
-#pragma unroll 2
-            for (int rep = 0; rep < every; ++rep) {
-                const float t = best[KK - 1];
-                const float2 eu = sub_f32x2(P, *reinterpret_cast<const unsigned long long*>(smem + up));
-                const float2 ed = sub_f32x2(P, *reinterpret_cast<const unsigned long long*>(smem + dn));
-                au = fabsf(eu.x) < t;
-                ad = fabsf(ed.x) < t;
-                const float du = fmaxf(fabsf(eu.x), fabsf(eu.y));
-                const float dd = fmaxf(fabsf(ed.x), fabsf(ed.y));
-                insert2<KK>(best, fminf(du, dd), fmaxf(du, dd));
-                up += au ? (int)sizeof(float2) : 0;
-                dn -= ad ? (int)sizeof(float2) : 0;
-            }
-            inblk = au || ad;  // a closed side stays closed: the threshold only shrinks
-        }
-        const bool aborted = steps > step_bound;
+        const uint2 found = lane_search<KK>(group * L.total, M, lw, gw, constant, switch_min, every);
+        const unsigned my_evals = found.x;
+        const bool aborted = found.y != 0u;
         group_sync(group);
 
         // ---- marginal counts and the digamma sum, evenly split over the group
