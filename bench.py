@@ -41,7 +41,7 @@ KSG_TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one l
 KSG_PRUNED_TRAFFIC_PER_VOLUME = (705.641e6 + 4.142e6) * 20
 KSG_BRUTE_TRAFFIC_PER_VOLUME = (705.845e6 + 4.089e6) * 20
 KSG_BLOCK_TRAFFIC_PER_VOLUME = (705.26e6 + 3.64e6) * 20
-KSG_LANES_TRAFFIC_PER_VOLUME = (704.32e6 + 3.37e6) * 20
+KSG_LANES_TRAFFIC_PER_VOLUME = (706.36e6 + 4.33e6) * 20
 KSG_SEARCHES = {  # name: (ndf constant name, kernel at k = 8, DRAM bytes per volume)
     "pruned": ("NDF_KSG_PRUNED", "ksg_pruned_kernel<9>", KSG_PRUNED_TRAFFIC_PER_VOLUME),
     "block": ("NDF_KSG_BLOCK", "ksg_block_kernel<9>", KSG_BLOCK_TRAFFIC_PER_VOLUME),

@@ -970,21 +970,22 @@ __global__ void __launch_bounds__(32 * kGroupWarps * kMaxGroupsPerCta, 1)
 //     least `switch_min` lanes wait or no lane is scanning, so the divergent code runs for
 //     many lanes at once;
 //   - every other lock step is the scan step of the block kernel for all lanes;
-//   - the marginal counts and the digamma sum (in fixed point: the same sum in any order, two
-//     integer adds for the slow FP64 pipe's one) follow in an evenly split pass over
-//     the stored eps (for KSG algorithm 2 after the marginal extents of each member's
+//   - the marginal counts (binary searches) and the digamma sum (in fixed point: the same sum in
+//     any order, two integer adds for the slow FP64 pipe's one) follow in an evenly split pass
+//     over the stored eps (for KSG algorithm 2 after the marginal extents of each member's
 //     k-NN set, found over the same blocks: block_extents).
 // What bounds it: the ALU pipe (the scan step's minima, maxima and compares issue at half
-// rate; 70 % busy at M = 1000, k = 8), then the shared-memory wavefronts of the lanes' scattered
-// reads (68 %) and the issue slots (62 %); 64,800 warp instructions per pair against 86,000 for
+// rate; 77 % busy at M = 1000, k = 8) and the L1 data pipe (74 %, the lanes' scattered reads of
+// shared memory 64 %); issue slots 65 %; 64,400 warp instructions per pair against 86,000 for
 // the sorted 64-rank blocks before.  250 x 352 x 20 vertices, M = 1000, k = 8: 167.5 ms before,
-// 133.5 - 139 ms now.
+// 130 - 133 ms now.
 // Members are handed out in the block kernel's task order (8 y-positions of 4 neighbouring
 // blocks per 32), so the lanes of a warp start on members of similar rank.  Shared memory per
 // pair: the block-sorted points, the sorted query column, one word per member (its query
 // value, then its rank, then eps) and the bitmaps (16 B x M + 5 B per block and 32 ranks);
-// the sorted reference values sit in shared memory once per CTA when all pairs share the
-// reference, else they are read from the staging buffer in global memory (L1).
+// for algorithm 1 the sorted reference values sit in shared memory once per CTA when all pairs share
+// the reference (and that costs no group, lane_plan), else they are read from the staging buffer in
+// global memory (L1).
 struct LaneCtl {
     unsigned long long item;
     unsigned long long pad;
